@@ -1419,6 +1419,7 @@ class EstimateRun {
 
   Plan p;
   Layout L, Lg;
+  Layout Lrow;  // L on the row-parallel kernels' own grid (untiled_gridx)
   int ds = 0, nv = 0, ng = 0, dso = 0, nvo = 0, ngo = 0, sub = 1, n_rec = 0;
   int64_t d_b = 0;
   bool store = false;
@@ -1471,7 +1472,7 @@ class EstimateRun {
   rdm_status init_block(char* w) {
     const BathPerm bp = hm.perm();  // bath vectors drawn in the caller's bath order
     CK(timed(kKInit, blk_b, [&] {
-      return launch_init_block(L, o->vec_dist, seed, o->first_vector, n_v, nullptr, d_vbuf, w, s, sub, &bp);
+      return launch_init_block(Lrow, o->vec_dist, seed, o->first_vector, n_v, nullptr, d_vbuf, w, s, sub, &bp);
     }));
     return RDM_OK;
   }
@@ -1507,6 +1508,12 @@ rdm_status EstimateRun::prepare(char* ws, size_t ws_bytes) {
   if (st != RDM_OK) return st;
   L = p.L;    // the recurrences (block size ds)
   Lg = p.Lg;  // the Gram view (groups of dso columns)
+  // The orthogonalisation and the starting block are bound by HBM and need about 8
+  // resident blocks per SM over all slices, whatever the tiled SpMM's one persistent block
+  // per SM and slice. On that grid a block of one slice (N = 24, 4 bath vectors) had 152
+  // blocks, and one of 200 slices (N = 16, 400 bath vectors) 30 400 of 3 rows a thread.
+  Lrow = L;
+  Lrow.gridx = untiled_gridx(L);
   ds = L.DS, nv = ds * ds, ng = L.n_groups();
   dso = 1 << hm.ns, nvo = dso * dso, ngo = Lg.n_groups();
   sub = p.single ? dso : 1;  // recurrences per bath vector
@@ -1641,9 +1648,9 @@ rdm_status EstimateRun::pass1() {
         CK(counted([&] {
           return launch_small_a(L, partials, MZ(j), d_ta + (size_t)(j - 1) * cstride, CW(j), d_flags, ls);
         }));
-        CK(timed(kKOrth1, blk_b * 3, [&] { return launch_orth(L, blk[cur], blk[nxt], CW(j), partials, ls); }));
+        CK(timed(kKOrth1, blk_b * 3, [&] { return launch_orth(Lrow, blk[cur], blk[nxt], CW(j), partials, ls); }));
         CK(counted([&] {
-          return launch_small_b(L, partials, MZ(j), d_tb + (size_t)(j - 1) * cstride, MZ(j + 1), CP(j + 1),
+          return launch_small_b(Lrow, partials, MZ(j), d_tb + (size_t)(j - 1) * cstride, MZ(j + 1), CP(j + 1),
                                 thr_abs_sq, thr_rel_sq, n_rec, d_flags, ls);
         }));
       }
@@ -1980,6 +1987,8 @@ rdm_status EstimateRun::finish_rest() {
         Ls.n_slices = Lgs.n_slices = nsl;
         Ls.B = nsl * L.Bs;
         Lgs.B = nsl * Lg.Bs;
+        Layout Lsr = Ls;
+        Lsr.gridx = untiled_gridx(Ls);  // the row-parallel kernels' grid, as Lrow
         const int g0 = s0 * L.groups_per_slice(), ngs = Ls.n_groups();
         const int g0o = s0 * Lg.groups_per_slice(), ngso = Lgs.n_groups();
         const size_t off = (size_t)s0 * slice_b, cs = (size_t)ngs * nv, cso = (size_t)ngso * nvo;
@@ -2021,11 +2030,11 @@ rdm_status EstimateRun::finish_rest() {
           const BathPerm bp = hm.perm();
           const char* vb = d_vbuf ? d_vbuf + (size_t)(g0 / sub) * (size_t)d_b * L.elem : nullptr;
           CK(timed(kKInit, bs, [&] {
-            return launch_init_block(Ls, o->vec_dist, seed, o->first_vector + g0 / sub, n_v - g0 / sub, nullptr, vb,
+            return launch_init_block(Lsr, o->vec_dist, seed, o->first_vector + g0 / sub, n_v - g0 / sub, nullptr, vb,
                                      wblk(1), s, sub, &bp);
           }));
         }
-        CK(timed(kKPsiInit, bs * (1 + nb), [&] { return launch_psi_init(Ls, wblk(1), psi, d_e, nb, s); }));
+        CK(timed(kKPsiInit, bs * (1 + nb), [&] { return launch_psi_init(Lsr, wblk(1), psi, d_e, nb, s); }));
         int j0 = 1;  // first step whose psi update is pending
         for (int j = 1; j < ke; ++j) {
           const int na = active(j);
@@ -2038,7 +2047,7 @@ rdm_status EstimateRun::finish_rest() {
           CK(timed(kKSpmm2, bs * (j >= 2 ? 3 : 2), [&] { return launch_spmm(Ls, kModePass2, sa, s); }));
           const int nf = mb > 1 ? 0 : na;  // betas updated by the orthogonalisation itself
           CK(timed(kKOrth2, bs * (3 + 2 * nf), [&] {
-            return launch_orth_psi(Ls, wblk(j), wblk(j + 1), CW(j) + (size_t)g0 * nv, psi,
+            return launch_orth_psi(Lsr, wblk(j), wblk(j + 1), CW(j) + (size_t)g0 * nv, psi,
                                    d_e + (size_t)j * p.nbc * cs, nf, s);
           }));
           if (mb > 1 && (j - j0 + 1 == mb || j == ke - 1)) {
@@ -2046,7 +2055,7 @@ rdm_status EstimateRun::finish_rest() {
             PsiBatch wb{};
             for (int a = 0; a < m; ++a) wb.w[a] = wblk(j0 + a + 1);
             CK(timed(kKPsiBatch, bs * (m + 2 * n0), [&] {
-              return launch_psi_batch(Ls, wb, m, psi, d_e + (size_t)j0 * p.nbc * cs, (size_t)p.nbc * cs, n0, s);
+              return launch_psi_batch(Lsr, wb, m, psi, d_e + (size_t)j0 * p.nbc * cs, (size_t)p.nbc * cs, n0, s);
             }));
             j0 = j + 1;
           }
