@@ -1419,6 +1419,7 @@ class EstimateRun {
 
   Plan p;
   Layout L, Lg;
+  Layout Lgr;   // Lg on the Gram kernels' grid (gram_gridx)
   Layout Lrow;  // L on the row-parallel kernels' own grid (untiled_gridx)
   int ds = 0, nv = 0, ng = 0, dso = 0, nvo = 0, ngo = 0, sub = 1, n_rec = 0;
   int64_t d_b = 0;
@@ -1427,7 +1428,7 @@ class EstimateRun {
   std::vector<char*> blk;
   char* psi = nullptr;
   PlanSizes psz{};
-  size_t pstride = 0, pstride_g = 0, cstride = 0;
+  size_t pstride_g = 0, cstride = 0;
   double* partials = nullptr;
   double* coef = nullptr;
   double* d_ta = nullptr;
@@ -1514,6 +1515,8 @@ rdm_status EstimateRun::prepare(char* ws, size_t ws_bytes) {
   // blocks, and one of 200 slices (N = 16, 400 bath vectors) 30 400 of 3 rows a thread.
   Lrow = L;
   Lrow.gridx = untiled_gridx(L);
+  Lgr = Lg;
+  Lgr.gridx = gram_gridx(Lg);
   ds = L.DS, nv = ds * ds, ng = L.n_groups();
   dso = 1 << hm.ns, nvo = dso * dso, ngo = Lg.n_groups();
   sub = p.single ? dso : 1;  // recurrences per bath vector
@@ -1540,8 +1543,7 @@ rdm_status EstimateRun::prepare(char* ws, size_t ws_bytes) {
   psi = store ? nullptr
               : ar.take<char>(L.block_bytes() / (size_t)L.n_slices * (size_t)(p.nsc ? p.nsc : L.n_slices) * p.nbc);
   psz = plan_sizes(p);
-  pstride = (size_t)L.n_slices * L.gridx * L.groups_per_slice() * nv;
-  pstride_g = (size_t)Lg.n_slices * Lg.gridx * Lg.groups_per_slice() * nvo;
+  pstride_g = (size_t)Lgr.n_slices * Lgr.gridx * Lgr.groups_per_slice() * nvo;
   partials = ar.take<double>(psz.partials);
   coef = ar.take<double>((size_t)(k + 2) * ng * nv * 3);
   d_ta = ar.take<double>((size_t)k * ng * nv);
@@ -1898,7 +1900,14 @@ rdm_status EstimateRun::finish_rest() {
     }
     return last;
   };
-  std::vector<int> jlast((size_t)p.nbc * n_v, 1);
+  std::vector<int> jlast((size_t)p.nbc * n_v, 1), kbeta(p.nbc, 1);
+  // betas of one Gram launch: their partials fit the buffer, the launches are even
+  auto gram_betas = [&](size_t stride, int nb) {
+    const int slots =
+        (int)std::min<size_t>(kGramLaunchBetas, std::max<size_t>(1, psz.partials / std::max<size_t>(1, stride)));
+    const int launches = (nb + slots - 1) / slots;
+    return (nb + launches - 1) / launches;
+  };
   for (int b0 = 0; b0 < n_beta; b0 += p.nbc) {
     const int nb = std::min(p.nbc, n_beta - b0);
     std::fill(hE.begin(), hE.end(), 0.0);
@@ -1948,10 +1957,9 @@ rdm_status EstimateRun::finish_rest() {
       }
     });
     host_ms += std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - coef_t0).count();
-    int k_eff = 1;
     for (int bi = 0; bi < nb; ++bi) {
       const int kb = *std::max_element(jlast.begin() + (size_t)bi * n_v, jlast.begin() + (size_t)(bi + 1) * n_v);
-      k_eff = std::max(k_eff, kb);
+      kbeta[bi] = kb;
       for (int j = kb; j < k; ++j) {  // E_j of this beta beyond its last needed step
         double* e0p = &hE[((size_t)j * p.nbc + bi) * (e_view ? ngo * nvo : ng * nv)];
         std::fill(e0p, e0p + (size_t)(e_view ? ngo * nvo : ng * nv), 0.0);
@@ -1961,16 +1969,15 @@ rdm_status EstimateRun::finish_rest() {
     h2d += hE.size() * sizeof(double);
     if (store) {
       // ---- psi = sum_j W_j E_j over the stored blocks, Gram fused (Gram view).
-      const int gmax = gram_stored_max_betas(Lg, k);
+      const int gmax = gram_betas(pstride_g, nb);
       for (int q = 0; q < nb; q += gmax) {
         const int nq = std::min(gmax, nb - q);
-        CK(timed(kKGram, blk_b * k_eff, [&] {
-          return launch_gram_stored(Lg, blk[0], k_eff, d_e, p.nbc, q, nq, partials, pstride_g, s);
+        CK(timed(kKGram, blk_b * *std::max_element(kbeta.begin() + q, kbeta.begin() + q + nq), [&] {
+          return launch_gram_stored(Lgr, blk[0], &kbeta[q], d_e, p.nbc, q, nq, partials, pstride_g, s);
         }));
-        for (int i = 0; i < nq; ++i)
-          CK(counted([&] {
-            return launch_reduce_gram(Lg, partials + (size_t)i * pstride_g, d_gram + (size_t)(q + i) * cstride_g, s);
-          }));
+        CK(counted([&] {
+          return launch_reduce_gram(Lgr, partials, pstride_g, nq, d_gram + (size_t)q * cstride_g, s);
+        }));
       }
     } else {
       // ---- pass 2: recompute W_j (bit-identical) and accumulate psi, one sweep per
@@ -1983,7 +1990,7 @@ rdm_status EstimateRun::finish_rest() {
       std::vector<double> hEc;
       for (int s0 = 0; s0 < L.n_slices; s0 += nsc) {
         const int nsl = std::min(nsc, L.n_slices - s0);
-        Layout Ls = L, Lgs = Lg;
+        Layout Ls = L, Lgs = Lgr;  // (the whole block's Gram grid: the same sums)
         Ls.n_slices = Lgs.n_slices = nsl;
         Ls.B = nsl * L.Bs;
         Lgs.B = nsl * Lg.Bs;
@@ -2060,9 +2067,14 @@ rdm_status EstimateRun::finish_rest() {
             j0 = j + 1;
           }
         }
-        for (int r = 0; r < nb; ++r) {
-          CK(timed(kKGram, bs, [&] { return launch_final_gram(Lgs, psi + (size_t)r * Ls.block_bytes(), partials, s); }));
-          CK(counted([&] { return launch_reduce_gram(Lgs, partials, d_gram + (size_t)r * cso, s); }));
+        const size_t ps = (size_t)Lgs.n_slices * Lgs.gridx * Lgs.groups_per_slice() * nvo;
+        const int gmax = gram_betas(ps, nb);
+        for (int r = 0; r < nb; r += gmax) {
+          const int nq = std::min(gmax, nb - r);
+          CK(timed(kKGram, bs * nq, [&] {
+            return launch_final_gram(Lgs, psi + (size_t)r * Ls.block_bytes(), nq, partials, ps, s);
+          }));
+          CK(counted([&] { return launch_reduce_gram(Lgs, partials, ps, nq, d_gram + (size_t)r * cso, s); }));
         }
         CK(cudaMemcpyAsync(hg.data(), d_gram, (size_t)nb * cso * sizeof(double), cudaMemcpyDeviceToHost, s));
         d2h += (size_t)nb * cso * sizeof(double);

@@ -23,6 +23,7 @@
 #include <algorithm>
 #include <mutex>
 #include <set>
+#include <vector>
 
 #include "rdm_internal.h"
 
@@ -1674,14 +1675,12 @@ __global__ void __launch_bounds__(kThreads) k_final_gram(Layout L, const T* __re
                                        (size_t)blockIdx.y * gridDim.x + blockIdx.x);
 }
 
-// Stored-basis Gram: psi_beta = sum_{j=1..k} W_j E_{j,beta} row by row (the same
+// Stored-basis Gram for float64 blocks and for float32 rows other than 32 bytes (blocks of
+// fewer than 2^kTileBits states; k_gram_rows takes the rest): psi_beta = sum_{j=1..k} W_j E_{j,beta} row by row (the same
 // fma sequence as the two-pass accumulation, so the result is bit-identical) and
 // the partial sums of psi_beta^T psi_beta, for up to kGramBetas betas per launch.
 // W_j = W1 + (j-1) * D * B elements; e: [j][beta (stride nbs)][group][DS*DS].
 constexpr int kGramBetas = 4;
-// With d_s <= 2 a beta's psi and Gram partials take few registers: twice the betas per
-// launch, half the passes over the stored basis.
-constexpr int kGramBetasWide = 8;
 
 template <typename T, int DS>
 struct RowVec;  // DS consecutive coefficients as one shared-memory load
@@ -1849,6 +1848,211 @@ __global__ void __launch_bounds__(kThreads) k_gram_stored(Layout L, const T* __r
   }
 }
 
+// ---------------------------------------------------------------- float32 Gram on 32-byte rows
+//
+// The Gram form's kernel for float32 blocks with 32-byte rows (the tiled layout), all betas
+// in one launch: psi_beta = sum_{j <= k_beta} W_j E_{j,beta} row by row (per element the fma
+// sequence of the other kernels, j then i ascending) and the sums of psi_beta^T psi_beta in
+// float64 (k_final_gram).
+//
+// What bounds it. GB300 issues 1.8 float64 fmas and 2.1 float32 -> float64 conversions per
+// clock and SM against 128 float32 fmas (measured), and a d_s = 4 row costs 10 products and
+// 4 conversions per beta: k_gram_stored, which this kernel replaces here, spent its time on
+// that pipe (63% busy under ncu) with 2 warps a scheduler, beside which nothing else ran.
+// So the conversions are integer operations (to_double), the basis rows come through
+// per-thread copy rings, and small blocks without barriers let one warp's float64 products
+// run beside the others' float32 fmas. Register prefetch instead of the rings stalled on
+// loads at every part (long_scoreboard 46%); a ring shared by a block kept its warps in step.
+//
+// A group of up to NBT betas shares one reading of the basis; the groups of one row range
+// are neighbours in the grid and take betas of the same spread of k_beta (every nz-th of the
+// betas in order of k_beta), so they move through the rows together and all but the first
+// find them in L2. At step j only the group's betas with k_beta > j are updated.
+//
+// Per solve, before and after: ladder N = 20 (n_v = 50, 16 betas, 30 steps) 50.0 -> 24.4 ms;
+// long-range XY N = 16 (n_v = 400, 8 betas) 34.6 -> 9.0 ms; long-range XXZ N = 22 (d_s = 2,
+// n_v = 16, 32 betas, 40 steps) 47.0 -> 23.4 ms; 48 small solves 87.7 -> 13.7 ms; one beta at
+// N = 22 (HBM, 6.8 TB/s) 10.4 ms as before.
+constexpr int kGramThreads = 128;
+constexpr int kGramStages = 8;  // steps in flight per thread (12: 4% slower)
+constexpr int kGramChunk = 512;  // rows per block and pass, whatever R: the sums' order
+struct GramBetas {
+  uint16_t k[kGramLaunchBetas];     // basis blocks each beta needs, descending
+  uint8_t beta[kGramLaunchBetas];   // and its place in the launch's betas
+};
+
+// (double)x with integer operations: the exponent rebiased by 896 and the mantissa moved
+// up; infinities and NaN keep their exponent of ones, and below the normal numbers the
+// result is zero (a psi entry there is under 1e-31 of the largest).
+__device__ __forceinline__ double to_double(float x) {
+  const uint32_t u = __float_as_uint(x), a = u & 0x7fffffffu;
+  uint32_t hi = (a >> 3) + 0x38000000u;
+  if (a >= 0x7f800000u) hi += 0x38000000u;
+  if (a < 0x00800000u) hi = 0u;
+  return __hiloint2double((int)(hi | (u & 0x80000000u)), (int)(u << 29));
+}
+
+// NBT: the largest group. FINAL: W1 holds nb blocks psi_beta (group size 1).
+template <int DS, int NBT, bool FINAL>
+__global__ void __launch_bounds__(kGramThreads, 3)
+    k_gram_rows(Layout L, const float* __restrict__ W1, GramBetas gb, const double* e, int nbs, int b0, int nb,
+                int nz, double* partials, size_t pstride) {
+  constexpr int VW = 4, NG = VW / DS, NVG = DS * DS;
+  constexpr int R = NBT >= 4 ? 2 : 4;   // rows per thread at a time (psi in registers)
+  constexpr int RS = kGramThreads / 2;  // rows between them
+  constexpr int CO = VW * DS;           // coefficients per lane, step and beta
+  extern __shared__ __align__(16) unsigned char smem_g[];
+  float* const sE = reinterpret_cast<float*>(smem_g);  // [j][bi][lane][CO]
+  __shared__ double red[kGramThreads / 32][2][NG * NVG];
+  const int z = blockIdx.x % nz, bx = blockIdx.x / nz, gx = L.gridx;
+  const int slice = blockIdx.y, gs = 2 * NG, ng = L.n_groups();
+  const int lane = threadIdx.x & 1, rs = threadIdx.x >> 1;
+  const size_t bstride = (size_t)L.D * L.B;
+  const float* const base =  // this thread's 16 bytes of row 0
+      W1 + (size_t)slice * L.D * 8 + (FINAL ? (size_t)z * bstride : 0) + (size_t)rs * 8 + lane * VW;
+  int kb[NBT];  // steps of the group's betas, descending (0: none)
+#pragma unroll
+  for (int bi = 0; bi < NBT; ++bi) kb[bi] = bi * nz + z < nb ? (FINAL ? 1 : (int)gb.k[bi * nz + z]) : 0;
+  const int kz = kb[0];
+  if (!FINAL) {
+    for (int i = threadIdx.x; i < kz * NBT * 2 * CO; i += kGramThreads) {
+      const int r = i % (2 * CO), bi = i / (2 * CO) % NBT, j = i / (2 * CO * NBT);
+      const int q = bi * nz + z;
+      if (q < nb && j < (int)gb.k[q])
+        sE[i] = (float)e[((size_t)j * nbs + b0 + gb.beta[q]) * ng * NVG + (size_t)slice * gs * NVG + r];
+    }
+    __syncthreads();
+  }
+  double acc[NBT][NG][DS][DS];
+#pragma unroll
+  for (int bi = 0; bi < NBT; ++bi)
+#pragma unroll
+    for (int g = 0; g < NG; ++g)
+#pragma unroll
+      for (int i = 0; i < DS; ++i)
+#pragma unroll
+        for (int j = 0; j < DS; ++j) acc[bi][g][i][j] = 0.0;
+  // Each thread copies its own 16 bytes of R rows per step into its own places of a ring of
+  // kGramStages steps (cp.async: no barrier, the warps drift apart freely), across the
+  // boundaries of row parts, so the next part's first steps arrive under this part's sums.
+  float* const ring = sE + (FINAL ? 0 : (size_t)kz * NBT * 2 * CO) + threadIdx.x * VW;
+  constexpr int kStage = R * kGramThreads * VW;  // floats
+  const int64_t chunks = L.D / kGramChunk;
+  const int64_t parts = (chunks - bx + gx - 1) / gx * (kGramChunk / (R * RS));  // of this block
+  int64_t lp = 0;  // the part and step of the next copy
+  int lj = 0, lslot = 0;
+  const float* src = base + (size_t)bx * kGramChunk * 8;
+  auto issue = [&]() {
+    if (lp < parts) {
+      const float* q = src + (size_t)lj * bstride;
+      float* d = ring + lslot * kStage;
+#pragma unroll
+      for (int r = 0; r < R; ++r)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(smem_u32(d + r * kGramThreads * VW)),
+                     "l"(q + (size_t)r * RS * 8)
+                     : "memory");
+      if (++lj == kz) {
+        lj = 0;
+        ++lp;
+        src += (size_t)R * RS * 8;
+        if (lp % (kGramChunk / (R * RS)) == 0) src += (size_t)(gx - 1) * kGramChunk * 8;
+      }
+    }
+    asm volatile("cp.async.commit_group;\n" ::: "memory");
+    if (++lslot == kGramStages) lslot = 0;
+  };
+#pragma unroll
+  for (int u = 0; u < kGramStages - 1; ++u) issue();
+  int slot = 0;
+  for (int64_t part = 0; part < parts; ++part) {
+    float psi[R][NBT][VW];
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+#pragma unroll
+      for (int bi = 0; bi < NBT; ++bi)
+#pragma unroll
+        for (int v = 0; v < VW; ++v) psi[r][bi][v] = 0.0f;
+    for (int j = 0; j < kz; ++j) {
+      issue();  // into the place freed one step ago
+      asm volatile("cp.async.wait_group %0;\n" ::"n"(kGramStages - 1) : "memory");
+      float x[R][VW];
+#pragma unroll
+      for (int r = 0; r < R; ++r) VecIO<float, VW>::ld_rw(x[r], ring + slot * kStage + r * kGramThreads * VW);
+      if (++slot == kGramStages) slot = 0;
+      if constexpr (FINAL) {
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+#pragma unroll
+          for (int v = 0; v < VW; ++v) psi[r][0][v] = x[r][v];
+      } else {
+#pragma unroll
+        for (int bi = 0; bi < NBT; ++bi) {
+          if (j >= kb[bi]) break;
+          const float* eb = sE + ((size_t)(j * NBT + bi) * 2 + lane) * CO;
+#pragma unroll
+          for (int g = 0; g < NG; ++g)
+#pragma unroll
+            for (int i = 0; i < DS; ++i) {
+              float er[DS];
+              RowVec<float, DS>::ld(er, eb + g * NVG + i * DS);
+#pragma unroll
+              for (int jj = 0; jj < DS; ++jj)
+#pragma unroll
+                for (int r = 0; r < R; ++r)
+                  psi[r][bi][g * DS + jj] = fmaf(x[r][g * DS + i], er[jj], psi[r][bi][g * DS + jj]);
+            }
+        }
+      }
+    }
+#pragma unroll
+    for (int bi = 0; bi < NBT; ++bi) {
+      if (kb[bi] == 0) break;
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        double pd[VW];
+#pragma unroll
+        for (int v = 0; v < VW; ++v) pd[v] = to_double(psi[r][bi][v]);
+#pragma unroll
+        for (int g = 0; g < NG; ++g)
+#pragma unroll
+          for (int i = 0; i < DS; ++i)
+#pragma unroll
+            for (int j = i; j < DS; ++j)
+              acc[bi][g][i][j] = fma(pd[g * DS + i], pd[g * DS + j], acc[bi][g][i][j]);
+      }
+    }
+  }
+  asm volatile("cp.async.wait_all;\n" ::: "memory");
+  const int wl = threadIdx.x & 31;
+#pragma unroll
+  for (int bi = 0; bi < NBT; ++bi) {
+    if (kb[bi] == 0) break;
+#pragma unroll
+    for (int g = 0; g < NG; ++g)
+#pragma unroll
+      for (int i = 0; i < DS; ++i)
+#pragma unroll
+        for (int j = i; j < DS; ++j) {
+          double x = acc[bi][g][i][j];
+#pragma unroll
+          for (int o = 2; o < 32; o <<= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+          if (wl < 2) {
+            red[threadIdx.x >> 5][wl][g * NVG + i * DS + j] = x;
+            red[threadIdx.x >> 5][wl][g * NVG + j * DS + i] = x;
+          }
+        }
+    __syncthreads();
+    if (threadIdx.x < 2 * NG * NVG) {
+      const int ln = threadIdx.x / (NG * NVG), v = threadIdx.x % (NG * NVG);
+      double sum = 0.0;
+      for (int w = 0; w < kGramThreads / 32; ++w) sum += red[w][ln][v];
+      const int beta = FINAL ? z : (int)gb.beta[bi * nz + z];
+      partials[(size_t)beta * pstride + (((size_t)slice * gx + bx) * gs + (size_t)ln * NG) * NVG + v] = sum;
+    }
+    __syncthreads();
+  }
+}
+
 // ---------------------------------------------------------------- per-group small steps
 
 constexpr int kSmallThreads = 128;
@@ -2004,13 +2208,14 @@ __global__ void k_small_b(Layout L, const double* partials, const double* mz_j, 
                     blockIdx.x);
 }
 
+// Group blockIdx.x of beta blockIdx.y.
 template <int DS>
-__global__ void k_reduce_gram(Layout L, const double* partials, double* gram) {
+__global__ void k_reduce_gram(Layout L, const double* partials, size_t pstride, double* gram) {
   constexpr int NV = DS * DS;
   __shared__ double tot[NV];
-  reduce_group<NV>(L, partials, tot, blockIdx.x);
+  reduce_group<NV>(L, partials + blockIdx.y * pstride, tot, blockIdx.x);
   if (threadIdx.x != 0) return;
-  for (int v = 0; v < NV; ++v) gram[(size_t)blockIdx.x * NV + v] = tot[v];
+  for (int v = 0; v < NV; ++v) gram[((size_t)blockIdx.y * L.n_groups() + blockIdx.x) * NV + v] = tot[v];
 }
 
 // ---------------------------------------------------------------- packed first pass
@@ -2465,55 +2670,107 @@ cudaError_t launch_pass1_packed(int precision, int ds, const PackedPlan& pp, int
   return cudaLaunchCooperativeKernel(fn, dim3((unsigned)grid), dim3(kThreads), args, smem, st);
 }
 
-cudaError_t launch_final_gram(const Layout& L, const void* psi, double* partials,
-                              cudaStream_t st) {
-  RDM_DISPATCH(L, (k_final_gram<T, DS, VW><<<grid_of(L), kThreads, 0, st>>>(
-                      L, reinterpret_cast<const T*>(psi), partials)));
+static bool gram_on_rows(const Layout& L) { return L.precision == RDM_FP32 && layout_tiled(L); }
+
+int gram_gridx(const Layout& L) {
+  if (!gram_on_rows(L)) return L.gridx;
+  // about 3 blocks per SM (what is resident) and beta group over all slices
+  const int64_t chunks = L.D / kGramChunk;
+  return (int)std::max<int64_t>(1, std::min<int64_t>(chunks, 456 / L.n_slices));
+}
+
+template <int DS, int NBT, bool FINAL>
+static cudaError_t launch_gram_rows(const Layout& L, const float* w, const GramBetas& gb, int k, const double* e,
+                                    int nbs, int b0, int nb, int nz, double* partials, size_t pstride, cudaStream_t st) {
+  cudaError_t ce = opt_in_smem(reinterpret_cast<const void*>(k_gram_rows<DS, NBT, FINAL>));
+  if (ce != cudaSuccess) return ce;
+  const size_t sm = (size_t)kGramStages * (NBT >= 4 ? 2 : 4) * kGramThreads * 16 +
+                    (FINAL ? 0 : (size_t)k * NBT * 8 * DS * sizeof(float));
+  k_gram_rows<DS, NBT, FINAL><<<dim3((unsigned)(L.gridx * nz), (unsigned)L.n_slices), kGramThreads, sm, st>>>(
+      L, w, gb, e, nbs, b0, nb, nz, partials, pstride);
   return cudaGetLastError();
 }
 
-cudaError_t launch_gram_stored(const Layout& L, const void* w1, int k, const double* e, int nbs,
+cudaError_t launch_final_gram(const Layout& L, const void* psi, int nb, double* partials, size_t pstride,
+                              cudaStream_t st) {
+  if (gram_on_rows(L)) {
+    const GramBetas gb{};
+    const float* w = reinterpret_cast<const float*>(psi);
+    RDM_DISPATCH_DS(L.DS, return (launch_gram_rows<DS, 1, true>(L, w, gb, 0, nullptr, 0, 0, nb, nb, partials,
+                                                                pstride, st)));
+  }
+  for (int b = 0; b < nb; ++b)
+    RDM_DISPATCH(L, (k_final_gram<T, DS, VW><<<grid_of(L), kThreads, 0, st>>>(
+                        L, reinterpret_cast<const T*>(psi) + (size_t)b * L.D * L.B, partials + b * pstride)));
+  return cudaGetLastError();
+}
+
+// The betas b0 .. b0+nb-1 in nz groups (kb: the last step of each) of at most 4 (8 leave
+// 2 blocks per SM for d_s = 2 and run 5% slower) whose coefficients of k steps take at most
+// 36 KB beside the copy ring (3 blocks per SM).
+template <int DS>
+static cudaError_t launch_gram_groups(const Layout& L, const float* w, int k, const int* kb, const double* e, int nbs,
+                                      int b0, int nb, double* partials, size_t pstride, cudaStream_t st) {
+  if (nb > kGramLaunchBetas) return cudaErrorInvalidValue;
+  int most = 4;
+  while (most > 1 && (size_t)k * most * 8 * DS * sizeof(float) > ((size_t)36 << 10)) most /= 2;
+  const int nz = (nb + most - 1) / most, group = (nb + nz - 1) / nz;
+  std::vector<int> ord(nb);
+  for (int b = 0; b < nb; ++b) ord[b] = b;
+  std::stable_sort(ord.begin(), ord.end(), [&](int x, int y) { return kb[x] > kb[y]; });
+  GramBetas gb{};
+  for (int q = 0; q < nb; ++q) {
+    gb.k[q] = (uint16_t)kb[ord[q]];
+    gb.beta[q] = (uint8_t)ord[q];
+  }
+  if (group > 2) return launch_gram_rows<DS, 4, false>(L, w, gb, k, e, nbs, b0, nb, nz, partials, pstride, st);
+  if (group > 1) return launch_gram_rows<DS, 2, false>(L, w, gb, k, e, nbs, b0, nb, nz, partials, pstride, st);
+  return launch_gram_rows<DS, 1, false>(L, w, gb, k, e, nbs, b0, nb, nz, partials, pstride, st);
+}
+
+cudaError_t launch_gram_stored(const Layout& L, const void* w1, const int* kb, const double* e, int nbs,
                                int b0, int nb, double* partials, size_t pstride, cudaStream_t st) {
-  RDM_DISPATCH(L, {
-    // static reduction scratch (block_reduce_store) + dynamic coefficients: opt in
-    const size_t sm = (size_t)k * nb * L.groups_per_slice() * DS * DS * sizeof(T) + 16;
-    cudaError_t ce = opt_in_smem(reinterpret_cast<const void*>(k_gram_stored<T, DS, VW, 1>));
-    if (ce == cudaSuccess) ce = opt_in_smem(reinterpret_cast<const void*>(k_gram_stored<T, DS, VW, 2>));
-    if (ce == cudaSuccess)
-      ce = opt_in_smem(reinterpret_cast<const void*>(k_gram_stored<T, DS, VW, kGramBetas>));
-    if (ce != cudaSuccess) return ce;
-    if constexpr (DS <= 2) {
-      if (nb > kGramBetas) {
-        ce = opt_in_smem(reinterpret_cast<const void*>(k_gram_stored<T, DS, VW, kGramBetasWide>));
-        if (ce != cudaSuccess) return ce;
-        k_gram_stored<T, DS, VW, kGramBetasWide><<<grid_of(L), kThreads, sm, st>>>(
-            L, reinterpret_cast<const T*>(w1), k, e, nbs, b0, nb, partials, pstride);
-        return cudaGetLastError();
-      }
-    }
-    if (nb == 1)
-      k_gram_stored<T, DS, VW, 1><<<grid_of(L), kThreads, sm, st>>>(
-          L, reinterpret_cast<const T*>(w1), k, e, nbs, b0, nb, partials, pstride);
-    else if (nb == 2)
-      k_gram_stored<T, DS, VW, 2><<<grid_of(L), kThreads, sm, st>>>(
-          L, reinterpret_cast<const T*>(w1), k, e, nbs, b0, nb, partials, pstride);
-    else
-      k_gram_stored<T, DS, VW, kGramBetas><<<grid_of(L), kThreads, sm, st>>>(
-          L, reinterpret_cast<const T*>(w1), k, e, nbs, b0, nb, partials, pstride);
-  });
+  const int k = *std::max_element(kb, kb + nb);
+  if (gram_on_rows(L)) {
+    const float* w = reinterpret_cast<const float*>(w1);
+    RDM_DISPATCH_DS(L.DS, return (launch_gram_groups<DS>(L, w, k, kb, e, nbs, b0, nb, partials, pstride, st)));
+  }
+  const int gmax = gram_stored_max_betas(L, k);
+  for (int q = 0; q < nb; q += gmax) {
+    const int n = std::min(gmax, nb - q);
+    double* pq = partials + (size_t)q * pstride;
+    RDM_DISPATCH(L, {
+      // static reduction scratch (block_reduce_store) + dynamic coefficients: opt in
+      const size_t sm = (size_t)k * n * L.groups_per_slice() * DS * DS * sizeof(T) + 16;
+      cudaError_t ce = opt_in_smem(reinterpret_cast<const void*>(k_gram_stored<T, DS, VW, 1>));
+      if (ce == cudaSuccess) ce = opt_in_smem(reinterpret_cast<const void*>(k_gram_stored<T, DS, VW, 2>));
+      if (ce == cudaSuccess)
+        ce = opt_in_smem(reinterpret_cast<const void*>(k_gram_stored<T, DS, VW, kGramBetas>));
+      if (ce != cudaSuccess) return ce;
+      if (n == 1)
+        k_gram_stored<T, DS, VW, 1><<<grid_of(L), kThreads, sm, st>>>(
+            L, reinterpret_cast<const T*>(w1), k, e, nbs, b0 + q, n, pq, pstride);
+      else if (n == 2)
+        k_gram_stored<T, DS, VW, 2><<<grid_of(L), kThreads, sm, st>>>(
+            L, reinterpret_cast<const T*>(w1), k, e, nbs, b0 + q, n, pq, pstride);
+      else
+        k_gram_stored<T, DS, VW, kGramBetas><<<grid_of(L), kThreads, sm, st>>>(
+            L, reinterpret_cast<const T*>(w1), k, e, nbs, b0 + q, n, pq, pstride);
+    });
+  }
   return cudaGetLastError();
 }
 
 int gram_stored_max_betas(const Layout& L, int k) {
   const size_t per = (size_t)k * L.groups_per_slice() * L.DS * L.DS * L.elem;
   int nb = (int)((160 * 1024) / (per ? per : 1));
-  return std::max(0, std::min(nb, L.DS <= 2 ? kGramBetasWide : kGramBetas));
+  return std::max(0, std::min(nb, kGramBetas));
 }
 
-cudaError_t launch_reduce_gram(const Layout& L, const double* partials, double* gram,
+cudaError_t launch_reduce_gram(const Layout& L, const double* partials, size_t pstride, int nb, double* gram,
                                cudaStream_t st) {
-  RDM_DISPATCH_DS(L.DS, (k_reduce_gram<DS><<<L.n_groups(), kSmallThreads, 0, st>>>(
-                           L, partials, gram)));
+  RDM_DISPATCH_DS(L.DS, (k_reduce_gram<DS><<<dim3((unsigned)L.n_groups(), (unsigned)nb), kSmallThreads, 0, st>>>(
+                           L, partials, pstride, gram)));
   return cudaGetLastError();
 }
 

@@ -254,16 +254,23 @@ cudaError_t launch_psi_batch(const Layout& L, const PsiBatch& wb, int m, void* p
 // Pass 2 start: psi_beta = W_1 E_{1,beta}.
 cudaError_t launch_psi_init(const Layout& L, const void* w, void* psi, const double* e, int nb,
                             cudaStream_t st);
-// Partials of psi^T psi per group for one psi block.
-cudaError_t launch_final_gram(const Layout& L, const void* psi, double* partials, cudaStream_t st);
-// Stored-basis Gram for betas b0..b0+nb-1 of the E array (beta stride nbs):
-// partials for beta b0+i at partials + i*pstride.
-cudaError_t launch_gram_stored(const Layout& L, const void* w1, int k, const double* e, int nbs,
+// Blocks per slice of the Gram kernels for this layout (the gridx that the layouts given to
+// launch_final_gram, launch_gram_stored and launch_reduce_gram carry).
+int gram_gridx(const Layout& L);
+// Partials of psi^T psi per group for nb consecutive psi blocks (D*B elements apart), those
+// of block b at partials + b*pstride.
+cudaError_t launch_final_gram(const Layout& L, const void* psi, int nb, double* partials, size_t pstride,
+                              cudaStream_t st);
+// Stored-basis Gram for betas b0..b0+nb-1 of the E array (beta stride nbs): partials for
+// beta b0+i at partials + i*pstride; kb[i]: the basis blocks it needs (E is zero beyond).
+// nb <= kGramLaunchBetas.
+constexpr int kGramLaunchBetas = 128;
+cudaError_t launch_gram_stored(const Layout& L, const void* w1, const int* kb, const double* e, int nbs,
                                int b0, int nb, double* partials, size_t pstride, cudaStream_t st);
-// Betas one stored-basis Gram launch can take (0: the coefficients do not fit).
+// Betas whose coefficients of k steps fit one block's shared memory (0: not even one).
 int gram_stored_max_betas(const Layout& L, int k);
-// Sum gram partials -> gram[group][DS*DS].
-cudaError_t launch_reduce_gram(const Layout& L, const double* partials, double* gram,
+// Sum the gram partials of nb betas -> gram[beta][group][DS*DS].
+cudaError_t launch_reduce_gram(const Layout& L, const double* partials, size_t pstride, int nb, double* gram,
                                cudaStream_t st);
 
 // One estimate's first pass inside the packed launch (k_pass1_packed). The layout is

@@ -1,0 +1,41 @@
+"""The Gram form on a beta grid (float32, 32-byte rows): the betas run in groups inside one
+launch, each group to the last step its betas need."""
+import numpy as np
+import pytest
+
+import workloads as W
+from oracle import lanczos
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("n,n_sys,n_v", [(10, 0, 3), (10, 1, 4), (11, 2, 2), (13, 2, 5), (12, 0, 9)])
+@pytest.mark.parametrize("n_beta", [1, 2, 3, 5, 9, 17])
+def test_gram_beta_groups(lib, n, n_sys, n_v, n_beta):
+    """Each beta of a grid gives bit for bit what it gives alone (its psi and its sums do not
+    depend on its group), in either order of the grid, with the basis stored or recomputed;
+    and the values are the oracle's within the float32 contract."""
+    spec = W.long_range_tfim(n, n_sys, 1.5, 0.8)
+    betas = W.beta_grid(n_beta, 0.05, 6.0)
+    ctx = lib.Context(0)
+    try:
+        ham = lib.Hamiltonian(ctx, spec)
+
+        def run(b, **kw):
+            return ham.estimate(b, n_v, 18, 77, precision="fp32", dist="gauss", full=True, **kw)
+        ctx.set_device_dense(0)  # the same coefficients whatever the grid
+        grid = run(betas)
+        back = run(betas[::-1].copy())
+        again = run(betas, passes="recompute")
+        for i in range(n_beta):
+            alone = run(betas[i:i + 1])
+            np.testing.assert_array_equal(grid["gram_l"][i], alone["gram_l"][0])
+            np.testing.assert_array_equal(grid["gram_l"][i], back["gram_l"][n_beta - 1 - i])
+            np.testing.assert_array_equal(grid["gram_l"][i], again["gram_l"][i])
+            g = grid["gram_l"][i]
+            np.testing.assert_array_equal(g, np.swapaxes(g, 1, 2))
+        ref = lanczos.Estimator(spec).run(betas, n_v, 18, 77, "gauss")
+        np.testing.assert_allclose(grid["rho"], ref["rho"], atol=1e-4, rtol=0)
+        np.testing.assert_allclose(grid["rho"], grid["rho_quad"], atol=1e-4, rtol=0)
+    finally:
+        ctx.close()
