@@ -282,7 +282,6 @@ static int tile_diag_layout(const std::vector<uint32_t>& mlo, uint32_t* dep, int
   return n;
 }
 
-// Groups the flip terms by m_high = mask >> kTileBits for the tiled SpMM.
 // The order in which the tiled SpMM walks the 2^b tiles of a slice: by the number of
 // set tile bits, and within one count by the ascending list of set bits in
 // lexicographic order (the simplicial order of the b-cube, whose prefixes have the
@@ -310,87 +309,144 @@ std::vector<uint32_t> tile_walk_order(int b) {
   return out;
 }
 
+// Sorts the flip terms into the tiled SpMM's tables (TiledTerms). Every mask has one bit (a
+// field) or two (a hop), so a term is placed by where its spins sit.
 void make_term_image(const HostModel& h, TermImage* img) {
-  std::map<uint32_t, std::vector<const FlipTerm*>> groups;
-  groups[0];  // pattern 0 always exists
-  for (const FlipTerm& f : h.flips) groups[f.mask >> kTileBits].push_back(&f);
-  // In-tile terms whose mask only touches a consumer thread's register rows (no bit
-  // below kTileRegShift) first: the SpMM applies them from registers.
-  auto& g0 = groups[0];
-  std::stable_partition(g0.begin(), g0.end(), [](const FlipTerm* f) {
-    return (f->mask & ((1u << kTileRegShift) - 1u)) == 0u;
-  });
-  img->n_reg0 = 0;
-  for (const FlipTerm* f : g0)
-    if ((f->mask & ((1u << kTileRegShift) - 1u)) == 0u) ++img->n_reg0;
-  std::vector<uint32_t> pat_high, pat_flags, term_low;
-  std::vector<int> pat_start;
-  std::vector<double> term_odd, term_even;
-  // Pattern 0 (in-tile terms) first, then partner tiles from the farthest (largest
-  // m_high, the likeliest L2 misses) to the nearest, so the slow copies enter the
-  // SpMM's copy ring early.
-  std::vector<std::pair<const uint32_t, std::vector<const FlipTerm*>>*> order;
-  for (auto& kv : groups) order.push_back(&kv);
-  std::sort(order.begin() + 1, order.end(), [](auto* x, auto* y) { return x->first > y->first; });
-  // Pairable partner tiles: one high spin h, and terms that each hop it with one spin
-  // l inside the tile with a parity-only coefficient (c_even = 0: XX + YY with
-  // J^x = J^y), the same set of l in every such group. For a given tile, a group whose
-  // h is down acts on the rows with l up and a group whose h is up on the rows with l
-  // down, so the SpMM consumes one of each together and every row takes exactly one of
-  // the two loads (no idle lanes). They go first, their terms in ascending l.
-  auto low_list = [](const std::vector<const FlipTerm*>& ts, std::vector<uint32_t>* out) -> bool {
+  constexpr uint32_t kRG = (1u << kTileRegShift) - 1u;  // row-group bits
+  struct Coef {
+    uint32_t flags = 0;
+    double c[7] = {};  // cf, co[3], ce[3]
+    void field(double v) {
+      flags |= kPatField;
+      c[0] += v;
+    }
+    void reg(uint32_t bit, double o, double e) {
+      const int a = __builtin_ctz(bit);
+      flags |= kPatReg << a;
+      c[1 + a] = o;
+      c[4 + a] = e;
+    }
+  };
+  struct Lane {
+    uint32_t low;
+    double o, e;
+  };
+  struct Pattern {
+    uint32_t high = 0;
+    Coef k;
+    std::vector<Lane> lanes;
+  };
+  std::map<uint32_t, Pattern> parts;  // by m_high != 0
+  std::map<uint32_t, Coef> groups;    // in-tile hops of a row-group spin with register spins
+  std::vector<Lane> own;
+  std::vector<double> reg_coef(16, 0.0);
+  img->reg_flags = 0;
+  img->all_uniform = 1;
+  for (const FlipTerm& f : h.flips) {
+    if (f.c_odd != f.c_even) img->all_uniform = 0;
+    const uint32_t high = f.mask >> kTileBits, low = f.mask & (uint32_t)(kTileRows - 1);
+    const uint32_t rg = low & kRG, reg = low >> kTileRegShift;
+    if (high) {
+      Pattern& P = parts[high];
+      P.high = high;
+      if (low == 0u) {
+        if (__builtin_popcount(high) == 1) {
+          P.k.field(f.c_odd);
+        } else {  // flat, two high spins
+          P.k.c[1] = f.c_odd;
+          P.k.c[4] = f.c_even;
+        }
+      } else if (reg) {
+        P.k.reg(reg, f.c_odd, f.c_even);
+      } else {
+        P.lanes.push_back(Lane{low, f.c_odd, f.c_even});
+      }
+    } else if (rg == 0u) {
+      img->reg_flags |= 1u << reg;
+      reg_coef[reg] = f.c_odd;
+      reg_coef[8 + reg] = f.c_even;
+    } else if (reg) {
+      groups[rg].reg(reg, f.c_odd, f.c_even);
+    } else {
+      own.push_back(Lane{low, f.c_odd, f.c_even});
+    }
+  }
+  // the field of a row-group spin joins the spin's group (the same loads)
+  for (size_t t = 0; t < own.size();) {
+    auto g = groups.find(own[t].low);
+    if (g != groups.end()) {
+      g->second.field(own[t].o);
+      own.erase(own.begin() + t);
+    } else {
+      ++t;
+    }
+  }
+  // Pairable patterns: one high spin without a field, hops that are all parity-only (c_even
+  // = 0: XX + YY with J^x = J^y), the same in-tile partners in every such pattern. For a
+  // given tile, a pattern whose spin is down acts on the rows whose in-tile spin is up and
+  // one whose spin is up on the others, so the SpMM consumes one of each together and every
+  // row takes exactly one of the two loads (no idle lanes).
+  auto partners_of = [&](const Pattern& P, std::vector<uint32_t>* out) -> bool {
     out->clear();
-    for (const FlipTerm* f : ts) {
-      const uint32_t low = f->mask & (uint32_t)(kTileRows - 1);
-      if (__builtin_popcount(low) != 1 || f->c_even != 0.0 || f->c_odd == 0.0) return false;
-      out->push_back(low);
+    if (__builtin_popcount(P.high) != 1 || (P.k.flags & kPatField)) return false;
+    for (int a = 0; a < 3; ++a)
+      if (P.k.flags & (kPatReg << a)) {
+        if (P.k.c[4 + a] != 0.0 || P.k.c[1 + a] == 0.0) return false;
+        out->push_back(1u << (kTileRegShift + a));
+      }
+    for (const Lane& t : P.lanes) {
+      if (t.e != 0.0 || t.o == 0.0) return false;
+      out->push_back(t.low);
     }
     std::sort(out->begin(), out->end());
-    return std::adjacent_find(out->begin(), out->end()) == out->end();
+    return !out->empty();
   };
-  int n_pair = 0;
-  {
-    std::vector<uint32_t> first, cur;
-    std::vector<char> is_pair(order.size(), 0);
-    bool have = false;
-    for (size_t q = 1; q < order.size(); ++q) {
-      if (__builtin_popcount(order[q]->first) != 1 || !low_list(order[q]->second, &cur)) continue;
-      if (!have) {
-        first = cur;
-        have = true;
+  std::vector<Pattern*> pairs, singles, flats;
+  std::vector<uint32_t> first, cur;
+  // From the farthest partner tile (largest m_high, the likeliest L2 miss) to the nearest,
+  // so the slow copies enter the SpMM's copy ring early.
+  for (auto it = parts.rbegin(); it != parts.rend(); ++it) {
+    Pattern& P = it->second;
+    std::sort(P.lanes.begin(), P.lanes.end(), [](const Lane& x, const Lane& y) { return x.low < y.low; });
+    if (P.lanes.empty() && !(P.k.flags & (kPatReg * 7u))) {
+      if (P.k.flags & kPatField) {  // a field alone
+        P.k.c[1] = P.k.c[4] = P.k.c[0];
+        P.k.flags = 0;
       }
-      if (cur == first) is_pair[q] = 1;
+      flats.push_back(&P);
+      continue;
     }
-    for (size_t q = 1; q < order.size(); ++q) n_pair += is_pair[q];
-    if (n_pair >= 2) {
-      std::vector<std::pair<const uint32_t, std::vector<const FlipTerm*>>*> head{order[0]}, tail;
-      for (size_t q = 1; q < order.size(); ++q) (is_pair[q] ? head : tail).push_back(order[q]);
-      for (size_t q = 1; q < head.size(); ++q)
-        std::sort(head[q]->second.begin(), head[q]->second.end(),
-                  [](const FlipTerm* x, const FlipTerm* y) { return x->mask < y->mask; });
-      order = head;
-      order.insert(order.end(), tail.begin(), tail.end());
-    } else {
-      n_pair = 0;
-    }
+    const bool ok = partners_of(P, &cur);
+    if (ok && first.empty()) first = cur;
+    (ok && cur == first ? pairs : singles).push_back(&P);
   }
-  for (auto* kvp : order) {
-    auto& kv = *kvp;
-    pat_high.push_back(kv.first);
-    pat_start.push_back((int)term_low.size());
-    uint32_t flags = 1u;
-    for (const FlipTerm* f : kv.second) {
-      const uint32_t low = f->mask & (uint32_t)(kTileRows - 1);
-      if (low) flags &= ~1u;
-      if (f->c_odd != 0.0) flags |= 2u;
-      if (f->c_even != 0.0) flags |= 4u;
-      term_low.push_back(low);
-      term_odd.push_back(f->c_odd);
-      term_even.push_back(f->c_even);
-    }
-    pat_flags.push_back(flags);
+  if (pairs.size() < 2) {
+    singles.insert(singles.begin(), pairs.begin(), pairs.end());
+    pairs.clear();
   }
-  pat_start.push_back((int)term_low.size());
+  std::vector<uint32_t> pat_high, pat_flags, lane_low, grp_low, grp_flags;
+  std::vector<int> pat_start;
+  std::vector<double> pat_coef, lane_coef, grp_coef;
+  auto put_lane = [&](const Lane& t) {
+    lane_low.push_back(t.low);
+    lane_coef.push_back(t.o);
+    lane_coef.push_back(t.e);
+  };
+  for (const Lane& t : own) put_lane(t);
+  for (const auto* list : {&pairs, &singles, &flats})
+    for (const Pattern* P : *list) {
+      pat_high.push_back(P->high);
+      pat_flags.push_back(P->k.flags);
+      pat_start.push_back((int)lane_low.size());
+      pat_coef.insert(pat_coef.end(), P->k.c, P->k.c + 7);
+      for (const Lane& t : P->lanes) put_lane(t);
+    }
+  pat_start.push_back((int)lane_low.size());
+  for (const auto& kv : groups) {
+    grp_low.push_back(kv.first);
+    grp_flags.push_back(kv.second.flags);
+    grp_coef.insert(grp_coef.end(), kv.second.c, kv.second.c + 7);
+  }
   // The diagonal split of the tiled SpMM: low table, K_0 terms, mixed groups by m_lo
   // (std::map keeps them in ascending m_lo, hence ascending m_lo >> kTileRegShift).
   std::vector<double> dg_low(kTileRows, 0.0);
@@ -432,25 +488,13 @@ void make_term_image(const HostModel& h, TermImage* img) {
   }
   img->dg_entries = tile_diag_layout(dg_mlo, &img->dg_dep, img->dg_off);
   const bool tiled = h.n >= kTileBits;
-  img->all_active = 1;
-  for (size_t q = 1; q < pat_flags.size(); ++q) {
-    const uint32_t f = pat_flags[q];
-    if ((f & 1u) && !((f & 2u) && (f & 4u))) img->all_active = 0;  // skipped by some tiles
-  }
-  // Every partner pattern one term with m_low = 0 and c_odd = c_even != 0 (a
-  // transverse field): the partner row of a row is the same row of the partner tile.
-  img->partners_flat = img->all_active;
-  for (size_t q = 1; q < pat_high.size(); ++q) {
-    const int t = pat_start[q];
-    if (pat_start[q + 1] - t != 1 || term_low[t] != 0u || term_odd[t] != term_even[t] || term_odd[t] == 0.0)
-      img->partners_flat = 0;
-  }
-  img->all_uniform = 1;
-  for (size_t t = 0; t < term_odd.size(); ++t)
-    if (term_odd[t] != term_even[t]) img->all_uniform = 0;
-  img->n_pat = tiled ? (int)pat_high.size() : 0;
-  img->n_pair = tiled ? n_pair : 0;
-  img->n_terms = tiled ? (int)term_low.size() : 0;
+  img->tiled = tiled ? 1 : 0;
+  img->n_part = (int)pat_high.size();
+  img->n_pair = (int)pairs.size();
+  img->n_single = (int)singles.size();
+  img->n_lane = (int)lane_low.size();
+  img->n_own = (int)own.size();
+  img->n_grp = (int)grp_low.size();
   auto& b = img->bytes;
   b.clear();
   auto put = [&](const void* src, size_t n) -> size_t {
@@ -464,9 +508,13 @@ void make_term_image(const HostModel& h, TermImage* img) {
   img->off_pat_high = put(pat_high.data(), pat_high.size() * 4);
   img->off_pat_start = put(pat_start.data(), pat_start.size() * 4);
   img->off_pat_flags = put(pat_flags.data(), pat_flags.size() * 4);
-  img->off_term_low = put(term_low.data(), term_low.size() * 4);
-  img->off_term_odd = put(term_odd.data(), term_odd.size() * 8);
-  img->off_term_even = put(term_even.data(), term_even.size() * 8);
+  img->off_pat_coef = put(pat_coef.data(), pat_coef.size() * 8);
+  img->off_lane_low = put(lane_low.data(), lane_low.size() * 4);
+  img->off_lane_coef = put(lane_coef.data(), lane_coef.size() * 8);
+  img->off_grp_low = put(grp_low.data(), grp_low.size() * 4);
+  img->off_grp_flags = put(grp_flags.data(), grp_flags.size() * 4);
+  img->off_grp_coef = put(grp_coef.data(), grp_coef.size() * 8);
+  img->off_reg_coef = put(reg_coef.data(), reg_coef.size() * 8);
   img->n_dg_groups = (int)dg_mlo.size();
   img->n_dg_terms = (int)dg_thi.size();
   img->off_dg_low = put(dg_low.data(), dg_low.size() * 8);
@@ -483,19 +531,25 @@ void bind_terms(const TermImage& img, char* dev, rdm_ham* ham) {
   ham->d_flips = reinterpret_cast<FlipTerm*>(dev + img.off_flips);
   ham->d_diags = reinterpret_cast<DiagTerm*>(dev + img.off_diags);
   TiledTerms& t = ham->tiled;
-  t.n_pat = img.n_pat;
+  t.ready = img.tiled;
+  t.n_part = img.n_part;
   t.n_pair = img.n_pair;
-  t.all_active = img.all_active;
-  t.partners_flat = img.partners_flat;
+  t.n_single = img.n_single;
+  t.n_lane = img.n_lane;
+  t.n_own = img.n_own;
+  t.n_grp = img.n_grp;
   t.all_uniform = img.all_uniform;
-  t.n_reg0 = img.n_reg0;
-  t.n_terms = img.n_terms;
+  t.reg_flags = img.reg_flags;
   t.pat_high = reinterpret_cast<const uint32_t*>(dev + img.off_pat_high);
   t.pat_start = reinterpret_cast<const int*>(dev + img.off_pat_start);
   t.pat_flags = reinterpret_cast<const uint32_t*>(dev + img.off_pat_flags);
-  t.term_low = reinterpret_cast<const uint32_t*>(dev + img.off_term_low);
-  t.term_odd = reinterpret_cast<const double*>(dev + img.off_term_odd);
-  t.term_even = reinterpret_cast<const double*>(dev + img.off_term_even);
+  t.pat_coef = reinterpret_cast<const double*>(dev + img.off_pat_coef);
+  t.lane_low = reinterpret_cast<const uint32_t*>(dev + img.off_lane_low);
+  t.lane_coef = reinterpret_cast<const double*>(dev + img.off_lane_coef);
+  t.grp_low = reinterpret_cast<const uint32_t*>(dev + img.off_grp_low);
+  t.grp_flags = reinterpret_cast<const uint32_t*>(dev + img.off_grp_flags);
+  t.grp_coef = reinterpret_cast<const double*>(dev + img.off_grp_coef);
+  t.reg_coef = reinterpret_cast<const double*>(dev + img.off_reg_coef);
   t.tile_order = reinterpret_cast<const uint32_t*>(dev + img.off_tile_order);
   TileDiag& d = t.dg;
   d.n_groups = img.n_dg_groups;
@@ -1119,7 +1173,7 @@ extern "C" rdm_status rdm_apply_hamiltonian(rdm_ham* ham, int precision, const v
   a.w = x;
   a.z = y;
   cudaStream_t s = ham->ctx->stream;
-  const bool tiled = layout_tiled(L) && ham->tiled.n_pat > 0;
+  const bool tiled = layout_tiled(L) && ham->tiled.ready;
   uint32_t* err = nullptr;
   if (tiled) {
     // The tiled SpMM reads the K table of the diagonal and reports copy-ring

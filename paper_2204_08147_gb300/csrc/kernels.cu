@@ -23,6 +23,7 @@
 #include <algorithm>
 #include <mutex>
 #include <set>
+#include <type_traits>
 #include <vector>
 
 #include "rdm_internal.h"
@@ -501,6 +502,19 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
 // table of the diagonal. Per tile the stage sequence is: own tile, each needed partner
 // tile, then the W_{j-1} tile (if any). Full barriers (count 1, transaction bytes)
 // and empty barriers (one arrival per consumer warp) order the ring.
+//
+// What bounds it: shared memory, whose 128 bytes per clock serve both the copies and the
+// consumers' 16-byte loads (ncu: loads 66% + copies 25% of the clocks for long-range XXZ
+// N = 22, 57% + 35% for the transverse field), and for the transverse field the copies out
+// of L2 (12.9 of the copy probe's 15.7 TB/s). Before, the consumers' instructions did:
+// 20 k per warp and XXZ tile, most of them scans over the patterns, address XORs and
+// per-term branches. Now the producers say with each stage what it is (ballots over the
+// patterns), every term is one address and constant offsets, the parity of a thread's rows
+// is a bit mask made once, and one set of loads serves all hops of a spin with the register
+// spins. Per launch, before and after: long-range XXZ N = 22 (n_v = 16) 4.17 -> 2.74 ms, N = 24
+// (n_v = 4) 4.95 -> 3.20 ms; long-range XY N = 16 (n_v = 400) 2.38 -> 1.38 ms (with the runs of
+// tiled_run_log); ladder N = 20 (n_v = 50) 1.58 -> 1.09 ms; transverse field N = 22 (n_v = 32)
+// 2.47 -> 2.38 ms.
 constexpr int kConsumerWarps = (kTileRows >> kTileRegBits) * kTiledLanes / 32;
 constexpr int kProducerWarps = 2;  // each issues the copies of every other ring slot
 constexpr int kTiledThreads = (kConsumerWarps + kProducerWarps) * 32;
@@ -511,48 +525,52 @@ __host__ __device__ inline uint32_t tiled_slot_bytes(int n_entries, int elem) {
   return kTileBytes + ((uint32_t)(tile_diag_stride(n_entries, elem) * elem) + 127u) / 128u * 128u;
 }
 
-// Shared-memory records of the tiled SpMM's term tables. A pattern record carries its
-// first term inline; `single` marks a pattern of one term with c_odd = c_even (one
-// coefficient for the whole tile), the common case of a transverse field.
+// Shared-memory records of the tiled SpMM's term tables (TiledTerms), in T.
 template <typename T>
-struct alignas(16) PatS {
-  uint32_t high;   // m_high: the partner tile is tile ^ high
-  uint32_t flags;  // bit0 uniform activity, bit1/bit2 some c_odd/c_even nonzero
-  int start, end;  // its terms
-  uint32_t low0;   // m_low of its first term
-  uint32_t single; // bit0: one term, c_odd = c_even; bit1: one term with m_low = 0
-  T c0;            // c_odd of its first term
-  T c1;            // c_even of its first term
+struct alignas(16) PatS {  // a partner pattern
+  uint32_t high;   // the partner tile is tile ^ high
+  uint32_t flags;  // kPatField, kPatReg
+  int start, end;  // its lane terms
+  T cf;            // field on its one high spin
+  T co[3], ce[3];  // hops with the spins of the register rows
 };
 template <typename T>
-struct alignas(16) TermS {
-  T co, ce;        // c_odd, c_even
-  uint32_t low;    // m_low
+struct alignas(16) LaneS {  // a term whose in-tile part moves the row group rg
+  T co, ce;
+  uint32_t off;  // element offset of m_low (XORed into a thread's row offset)
+  uint32_t low;  // m_low
 };
+template <typename T>
+struct alignas(16) GrpS {  // in-tile terms of one row-group spin l: field, hops with register spins
+  uint32_t off, low, flags;
+  T cf;
+  T co[3], ce[3];
+};
+// What the producer says of a ring stage: the own tile's holds its index and the number
+// of the tile's partner stages, a partner stage's its pattern (+ kJoint for the first of an
+// opposite-spin pair) and, for a flat pattern, its coefficient in this tile.
+template <typename T>
+struct alignas(16) StageS {
+  int what;
+  uint32_t tile;  // the own tile's index
+  T c;
+};
+constexpr int kJoint = 1 << 16;
 
 template <typename T>
-__host__ __device__ inline size_t tiled_smem_bytes(int n_pat, int n_terms, int n_entries, int stages) {
+__host__ __device__ inline size_t tiled_smem_bytes(int n_part, int n_lane, int n_grp, int n_entries, int stages) {
   size_t off = (size_t)stages * tiled_slot_bytes(n_entries, (int)sizeof(T));
   off += 2 * kMaxStages * 8 + 64;                  // full/empty barriers, control
   off += 2 * 8 * 16 * sizeof(T);                   // mixing coefficients of the lanes
   off += (size_t)kConsumerWarps * kTiledLanes * 16 * 8;  // reduction scratch
   off = (off + 15) / 16 * 16;
-  off += (size_t)n_pat * sizeof(PatS<T>);          // pattern records
+  off += kMaxStages * sizeof(StageS<T>);
+  off += (size_t)n_part * sizeof(PatS<T>);
+  off += (size_t)n_grp * sizeof(GrpS<T>);
+  off += (size_t)n_lane * sizeof(LaneS<T>);
+  off += 16 * sizeof(T);                           // hops and fields of the register rows
   off += (size_t)kTileRows * sizeof(T);            // low table of the diagonal
-  off += (size_t)n_terms * sizeof(TermS<T>);       // term records
   return off + 64;
-}
-
-// First pattern >= p that tile tix needs (uniform patterns may be inactive).
-template <typename T>
-__device__ __forceinline__ int tiled_next(int p, int npat, uint32_t tix, const PatS<T>* pat) {
-  for (; p < npat; ++p) {
-    const uint32_t f = pat[p].flags;
-    if (!(f & 1u)) return p;
-    const bool odd = (__popc(tix & pat[p].high) & 1) != 0;
-    if (odd ? (f & 2u) : (f & 4u)) return p;
-  }
-  return p;
 }
 
 __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
@@ -578,245 +596,77 @@ __device__ __forceinline__ bool ring_wait(uint64_t* bar, uint32_t parity, volati
   return false;
 }
 
-// In-tile flip whose partner rows belong to the same thread: the thread's rows
-// rg + RG m (m = 0..7) form a subcube over the top three tile bits, so a mask with
-// no bit below log2(RG) maps row m to row m ^ K of the same thread.
-template <int K, int RG, bool UNI, typename T, int VW, int RPT>
-__device__ __forceinline__ void reg_flip(T (&y)[RPT][VW], const T (&xo)[RPT][VW], int rg, uint32_t ml,
-                                         T co, T ce) {
-  if constexpr (K >= RPT) return;
-  if (UNI || co == ce) {
+// Rows of a consumer thread: row rg + RG m (m = 0..RPT-1) of a tile sits at element offset
+// rgoff + m * kStep (rgoff = rg * BS + lane * VW, kStep = RG * BS). Under a mask m_low in the
+// row-group bits its partner rows sit at (rgoff ^ m_low * BS) + m * kStep: one address and
+// constant offsets. A mask bit in the register rows only renames m.
+template <int STEP, typename T, int VW, int RPT>
+__device__ __forceinline__ void load_rows(T (&x)[RPT][VW], const T* p) {
 #pragma unroll
-    for (int m = 0; m < RPT; ++m)
-#pragma unroll
-      for (int v = 0; v < VW; ++v) y[m][v] = fma(co, xo[(m ^ K) & (RPT - 1)][v], y[m][v]);
-    return;
-  }
-#pragma unroll
-  for (int m = 0; m < RPT; ++m) {
-    const uint32_t r = (uint32_t)(rg + RG * m);
-    const T c = (__popc(r & ml) & 1) ? co : ce;
-#pragma unroll
-    for (int v = 0; v < VW; ++v) y[m][v] = fma(c, xo[(m ^ K) & (RPT - 1)][v], y[m][v]);
-  }
+  for (int m = 0; m < RPT; ++m) VecIO<T, VW>::ld_rw(x[m], p + m * STEP);
 }
-
-// Rows of a consumer thread and their partners: row rg + RG m (m = 0..7) of a tile sits
-// at element offset rgoff + m * kStep (rgoff = rg * BS + lane * VW, kStep = RG * BS,
-// both powers of two apart), so under an in-tile mask ml = (mh << log2 RG) | mlow its
-// partner row rg ^ mlow + RG (m ^ mh) sits at (rgoff ^ mlow * BS | mh * kStep) ^ m * kStep.
-// With mh = 0 that is a base plus a constant per row.
-template <int RG, int BS>
-__device__ __forceinline__ int partner_base(int rgoff, uint32_t ml) {
-  return (rgoff ^ (int)((ml & (uint32_t)(RG - 1)) * BS)) | (int)((ml / RG) * (uint32_t)(RG * BS));
-}
-
-// Rows m and m ^ K (K a register-row bit of mh) of this thread for a parity-only term:
-// the pair's active row a (parity p0 ^ parity(a & mh) selects the nonzero coefficient)
-// loads its partner row once; y[a] += c * partner, y[other] += 0 * partner.
-template <int K, typename T, int VW, int RPT>
-__device__ __forceinline__ void pair_rows(T (&y)[RPT][VW], const T* P, int x, int kStep, uint32_t mh, uint32_t p0,
-                                          T co, T ce) {
-  if constexpr (K >= RPT) return;
-  const T c = co != (T)0 ? co : ce;
-  const uint32_t want = co != (T)0 ? 1u : 0u;  // the parity with the nonzero coefficient
-  if (mh == (uint32_t)K) {
-    // one register-row bit in the mask: every pair (m, m ^ K) with m & K = 0 has its
-    // active row on the same side, so the side, its coefficients and the partner
-    // offset are chosen once
-    const bool lo = p0 == want;
-    const T cl = lo ? c : (T)0, ch = lo ? (T)0 : c;
-    const int xs = lo ? x : (x ^ (K * kStep));
+// y += c x; float32 two columns at a time (fma.rn.f32x2 rounds each as fmaf does; few-term
+// models 5% faster, but the flat partner tiles below 1.5% slower)
+template <typename T, int VW>
+__device__ __forceinline__ void axpy(T (&y)[VW], T c, const T (&x)[VW]) {
+  if constexpr (sizeof(T) == 4) {
 #pragma unroll
-    for (int m = 0; m < RPT; ++m) {
-      if (m & K) continue;
-      T xp[VW];
-      VecIO<T, VW>::ld_rw(xp, P + (xs ^ (m * kStep)));
-#pragma unroll
-      for (int v = 0; v < VW; ++v) {
-        y[m][v] = fma(cl, xp[v], y[m][v]);
-        y[m ^ K][v] = fma(ch, xp[v], y[m ^ K][v]);
-      }
-    }
-    return;
-  }
-#pragma unroll
-  for (int m = 0; m < RPT; ++m) {
-    if (m & K) continue;
-    const bool lo = ((p0 ^ (uint32_t)__popc((uint32_t)m & mh)) & 1u) == want;
-    const int a = lo ? m : (m ^ K);
-    T xp[VW];
-    VecIO<T, VW>::ld_rw(xp, P + (x ^ (a * kStep)));
-    const T cl = lo ? c : (T)0, ch = lo ? (T)0 : c;
-#pragma unroll
-    for (int v = 0; v < VW; ++v) {
-      y[m][v] = fma(cl, xp[v], y[m][v]);
-      y[m ^ K][v] = fma(ch, xp[v], y[m ^ K][v]);
-    }
-  }
-}
-
-// y[m] += c * P[row m ^ ml] for one term whose coefficient depends on the parity of
-// (row0 + row) & mparity (c_odd / c_even), rows of this thread.
-// UNI: every term of the Hamiltonian has c_odd = c_even (a separate instantiation,
-// so the parity-dependent code below is not compiled into it).
-template <typename T, int VW, int RPT, int RG, int BS, bool UNI>
-__device__ __forceinline__ void apply_term(T (&y)[RPT][VW], int rgoff, int rg, const T* P, uint32_t ml,
-                                           uint32_t mparity, T co, T ce, uint32_t row0) {
-  constexpr int kStep = RG * BS;
-  const int x = partner_base<RG, BS>(rgoff, ml);
-  const bool flat = ml < (uint32_t)RG;  // mh = 0: partner offsets x + m * kStep
-  if (UNI || co == ce) {
-    if (flat) {
-#pragma unroll
-      for (int m = 0; m < RPT; ++m) {
-        T xp[VW];
-        VecIO<T, VW>::ld_rw(xp, P + x + m * kStep);
-#pragma unroll
-        for (int v = 0; v < VW; ++v) y[m][v] = fma(co, xp[v], y[m][v]);
-      }
-    } else {
-#pragma unroll
-      for (int m = 0; m < RPT; ++m) {
-        T xp[VW];
-        VecIO<T, VW>::ld_rw(xp, P + (x ^ (m * kStep)));
-#pragma unroll
-        for (int v = 0; v < VW; ++v) y[m][v] = fma(co, xp[v], y[m][v]);
-      }
-    }
-  } else if constexpr (!UNI) {
-    // Row row0 + rg + RG m is row0 | rg | m << log2(RG) (disjoint bits), so its parity
-    // under mparity is p0 (that of row0 | rg) xor the parity of m & mh. With mh = 0 the
-    // coefficient is the same for all of this thread's rows: one test per term.
-    const uint32_t mh = (mparity / (uint32_t)RG) & (uint32_t)(RPT - 1);
-    const uint32_t p0 = (uint32_t)__popc((row0 + (uint32_t)rg) & mparity) & 1u;
-    if (mh == 0u) {
-      // the same coefficient for all of this thread's rows; where it differs across the
-      // warp's lanes they all run the term (a zero coefficient on the others) rather
-      // than diverge, and a warp none of whose lanes has it skips the term
-      const T c = p0 ? co : ce;
-      if (__any_sync(0xffffffffu, c != (T)0)) {
-#pragma unroll
-        for (int m = 0; m < RPT; ++m) {
-          T xp[VW];
-          VecIO<T, VW>::ld_rw(xp, P + (x ^ (m * kStep)));
-#pragma unroll
-          for (int v = 0; v < VW; ++v) y[m][v] = fma(c, xp[v], y[m][v]);
-        }
-      }
-    } else if (co == (T)0 || ce == (T)0) {
-      // Parity-only coefficient (one of c_odd, c_even zero, e.g. XX + YY with J^x = J^y):
-      // rows m and m ^ hb (hb the lowest bit of mh) have opposite parities, so exactly one
-      // of each such pair is active. One load serves the pair: the active row's partner,
-      // added to the active row (the other row's product is with zero).
-      switch (mh & (0u - mh)) {
-        case 1u: pair_rows<1, T, VW, RPT>(y, P, x, kStep, mh, p0, co, ce); break;
-        case 2u: pair_rows<2, T, VW, RPT>(y, P, x, kStep, mh, p0, co, ce); break;
-        default: pair_rows<4, T, VW, RPT>(y, P, x, kStep, mh, p0, co, ce); break;
-      }
-    } else {
-#pragma unroll
-      for (int m = 0; m < RPT; ++m) {
-        const T c = ((p0 ^ (uint32_t)__popc((uint32_t)m & mh)) & 1u) ? co : ce;
-        if (c != (T)0) {
-          T xp[VW];
-          VecIO<T, VW>::ld_rw(xp, P + (x ^ (m * kStep)));
-#pragma unroll
-          for (int v = 0; v < VW; ++v) y[m][v] = fma(c, xp[v], y[m][v]);
-        }
-      }
-    }
-  }
-}
-
-// Two uniform-coefficient terms at once (loads of both issued before their FMAs).
-template <typename T, int VW, int RPT, int RG, int BS>
-__device__ __forceinline__ void apply2_uniform(T (&y)[RPT][VW], int rgoff, const T* PA, uint32_t mlA, T cA,
-                                               const T* PB, uint32_t mlB, T cB) {
-  constexpr int kStep = RG * BS;
-  const int xa = partner_base<RG, BS>(rgoff, mlA), xb = partner_base<RG, BS>(rgoff, mlB);
-  if (mlA < (uint32_t)RG && mlB < (uint32_t)RG) {
-#pragma unroll
-    for (int m = 0; m < RPT; ++m) {
-      T a[VW], b[VW];
-      VecIO<T, VW>::ld_rw(a, PA + xa + m * kStep);
-      VecIO<T, VW>::ld_rw(b, PB + xb + m * kStep);
-#pragma unroll
-      for (int v = 0; v < VW; ++v) y[m][v] = fma(cB, b[v], fma(cA, a[v], y[m][v]));
-    }
+    for (int v = 0; v < VW; v += 2)
+      asm("{\n .reg .b64 c, x, y;\n mov.b64 c, {%2, %2};\n mov.b64 x, {%3, %4};\n mov.b64 y, {%0, %1};\n"
+          " fma.rn.f32x2 y, c, x, y;\n mov.b64 {%0, %1}, y;\n}\n"
+          : "+f"(y[v]), "+f"(y[v + 1])
+          : "f"(c), "f"(x[v]), "f"(x[v + 1]));
   } else {
 #pragma unroll
-    for (int m = 0; m < RPT; ++m) {
-      T a[VW], b[VW];
-      VecIO<T, VW>::ld_rw(a, PA + (xa ^ (m * kStep)));
-      VecIO<T, VW>::ld_rw(b, PB + (xb ^ (m * kStep)));
-#pragma unroll
-      for (int v = 0; v < VW; ++v) y[m][v] = fma(cB, b[v], fma(cA, a[v], y[m][v]));
-    }
+    for (int v = 0; v < VW; ++v) y[v] = fma(c, x[v], y[v]);
   }
 }
-
-// Pairable partner tiles (TiledTerms::n_pair): for a tile, the groups of one high spin h
-// whose h is down (zm, bit q = pattern q + 1) and up (om). The i-th stage of the block:
-// down and up groups alternate (z_0, o_0, z_1, o_1, ..), then the rest of the longer list.
-__device__ __forceinline__ int pair_pattern(int i, uint32_t zm, uint32_t om) {
-  const int nz = __popc(zm), no = __popc(om), mn = nz < no ? nz : no;
-  uint32_t m;
-  int k;
-  if (i < 2 * mn) {
-    m = (i & 1) ? om : zm;
-    k = i >> 1;
-  } else {
-    m = nz > no ? zm : om;
-    k = i - mn;
-  }
-  for (; k > 0; --k) m &= m - 1u;
-  return __ffs((int)m);
-}
-
-// Term i of both groups hops the same in-tile spin l with h (parity-only coefficient,
-// active where l and h differ): with h down in PZ and up in PO, a row whose spin l is up
-// takes PZ's term and a row whose spin l is down PO's, so every row loads once per l.
-template <int K, typename T, int VW, int RPT>
-__device__ __forceinline__ void paired_reg(T (&y)[RPT][VW], const T* PZ, const T* PO, int x, int kStep, T cz,
-                                           T co) {
-  if constexpr (K >= RPT) return;
+// Whether a coefficient is not +0, by its bits (a float64 compare would take the narrow
+// float64 pipe).
+__device__ __forceinline__ bool in_use(float c) { return __float_as_int(c) != 0; }
+__device__ __forceinline__ bool in_use(double c) { return (__double2hiint(c) | __double2loint(c)) != 0; }
+// y[m] += c * (row m of p)
+template <int STEP, typename T, int VW, int RPT>
+__device__ __forceinline__ void rows_fma(T (&y)[RPT][VW], const T* p, T c) {
 #pragma unroll
   for (int m = 0; m < RPT; ++m) {
-    T xp[VW];
-    VecIO<T, VW>::ld_rw(xp, ((m & K) ? PZ : PO) + (x ^ (m * kStep)));
-    const T c = (m & K) ? cz : co;
-#pragma unroll
-    for (int v = 0; v < VW; ++v) y[m][v] = fma(c, xp[v], y[m][v]);
+    T x[VW];
+    VecIO<T, VW>::ld_rw(x, p + m * STEP);
+    axpy(y[m], c, x);
   }
 }
-template <typename T, int VW, int RPT, int RG, int BS>
-__device__ __forceinline__ void apply_paired(T (&y)[RPT][VW], int rgoff, int rg, const T* PZ, const T* PO,
-                                             const TermS<T>* tz, const TermS<T>* to, int nt) {
-  constexpr int kStep = RG * BS;
-  for (int i = 0; i < nt; ++i) {
-    const uint32_t ml = tz[i].low;
-    const T cz = tz[i].co, co = to[i].co;
-    const int x = partner_base<RG, BS>(rgoff, ml);
-    if (ml < (uint32_t)RG) {  // spin l is a bit of rg: the same for all of this thread's rows
-      const bool up = ((uint32_t)rg & ml) != 0u;
-      const T* P = up ? PZ : PO;
-      const T c = up ? cz : co;
+// y[m] += cA * (row m of a) + cB * (row m of b), the loads of both before their fmas
+template <int STEP, typename T, int VW, int RPT>
+__device__ __forceinline__ void rows_fma2(T (&y)[RPT][VW], const T* a, T cA, const T* b, T cB) {
 #pragma unroll
-      for (int m = 0; m < RPT; ++m) {
-        T xp[VW];
-        VecIO<T, VW>::ld_rw(xp, P + x + m * kStep);
+  for (int m = 0; m < RPT; ++m) {
+    T u[VW], w[VW];
+    VecIO<T, VW>::ld_rw(u, a + m * STEP);
+    VecIO<T, VW>::ld_rw(w, b + m * STEP);
 #pragma unroll
-        for (int v = 0; v < VW; ++v) y[m][v] = fma(c, xp[v], y[m][v]);
-      }
-    } else {
-      switch (ml / (uint32_t)RG) {
-        case 1u: paired_reg<1, T, VW, RPT>(y, PZ, PO, x, kStep, cz, co); break;
-        case 2u: paired_reg<2, T, VW, RPT>(y, PZ, PO, x, kStep, cz, co); break;
-        default: paired_reg<4, T, VW, RPT>(y, PZ, PO, x, kStep, cz, co); break;
-      }
-    }
+    for (int v = 0; v < VW; ++v) y[m][v] = fma(cB, w[v], fma(cA, u[v], y[m][v]));
   }
+}
+// y[m] += c * x[m ^ K] on the rows m whose parity under K is ODD
+template <int K, int ODD, typename T, int VW, int RPT>
+__device__ __forceinline__ void reg_half(T (&y)[RPT][VW], const T (&x)[RPT][VW], T c) {
+#pragma unroll
+  for (int m = 0; m < RPT; ++m) {
+    if ((((m & K) ^ ((m & K) >> 1) ^ ((m & K) >> 2)) & 1) != ODD) continue;
+    axpy(y[m], c, x[m ^ K]);
+  }
+}
+// The coefficients of both halves are the same across the warp (skipped when zero) ...
+template <int K, typename T, int VW, int RPT>
+__device__ __forceinline__ void reg_uniform(T (&y)[RPT][VW], const T (&x)[RPT][VW], T c_even, T c_odd) {
+  if (in_use(c_even)) reg_half<K, 0>(y, x, c_even);
+  if (in_use(c_odd)) reg_half<K, 1>(y, x, c_odd);
+}
+// ... or differ between its lanes (a half is skipped when it is zero on all of them).
+template <int K, typename T, int VW, int RPT>
+__device__ __forceinline__ void reg_lanes(T (&y)[RPT][VW], const T (&x)[RPT][VW], T c_even, T c_odd) {
+  if (__any_sync(0xffffffffu, in_use(c_even))) reg_half<K, 0>(y, x, c_even);
+  if (__any_sync(0xffffffffu, in_use(c_odd))) reg_half<K, 1>(y, x, c_odd);
 }
 
 // Diagonal of H on this thread's RPT rows rg + RG m of a tile, from the tile's A-table
@@ -864,7 +714,7 @@ __global__ void __launch_bounds__(kTiledThreads, 1) k_spmm_tiled(Layout L, SpmmA
   static_assert((1 << RGL) == RG && RGL == kTileRegShift, "row groups are the low tile bits");
   extern __shared__ __align__(128) unsigned char smem[];
   const TiledTerms& tt = a.tiled;
-  const int npat = tt.n_pat, nterm = tt.n_terms, npair = tt.n_pair;
+  const int npart = tt.n_part, nlane = tt.n_lane, npair = tt.n_pair, nsingle = tt.n_single;
   const int hstride = tile_diag_stride(tt.dg.n_entries, (int)sizeof(T));
   const uint32_t kSlotBytes = tiled_slot_bytes(tt.dg.n_entries, (int)sizeof(T));
   unsigned char* const ring = smem;
@@ -876,32 +726,49 @@ __global__ void __launch_bounds__(kTiledThreads, 1) k_spmm_tiled(Layout L, SpmmA
   double* const red = reinterpret_cast<double*>(s_cp + 8 * 16);
   size_t off = (size_t)(reinterpret_cast<unsigned char*>(red + kConsumerWarps * kTiledLanes * 16) - smem);
   off = (off + 15) / 16 * 16;
-  PatS<T>* const pat = reinterpret_cast<PatS<T>*>(smem + off);
-  T* const s_low = reinterpret_cast<T*>(pat + npat);
-  TermS<T>* const term = reinterpret_cast<TermS<T>*>(s_low + kTileRows);
+  StageS<T>* const stage = reinterpret_cast<StageS<T>*>(smem + off);
+  PatS<T>* const pat = reinterpret_cast<PatS<T>*>(stage + kMaxStages);
+  GrpS<T>* const grp = reinterpret_cast<GrpS<T>*>(pat + npart);
+  LaneS<T>* const lanet = reinterpret_cast<LaneS<T>*>(grp + tt.n_grp);
+  T* const s_reg = reinterpret_cast<T*>(lanet + nlane);  // [8] c_odd, [8] c_even
+  T* const s_low = s_reg + 16;
 
-  for (int i = threadIdx.x; i < npat; i += blockDim.x) {
+  for (int i = threadIdx.x; i < npart; i += blockDim.x) {
     PatS<T> r;
+    const double* c = tt.pat_coef + (size_t)i * 7;
     r.high = tt.pat_high[i];
     r.flags = tt.pat_flags[i];
     r.start = tt.pat_start[i];
     r.end = tt.pat_start[i + 1];
-    const bool any = r.start < r.end;
-    r.low0 = any ? tt.term_low[r.start] : 0u;
-    r.c0 = any ? (T)tt.term_odd[r.start] : (T)0;
-    r.c1 = any ? (T)tt.term_even[r.start] : (T)0;
-    const bool one = r.end - r.start == 1;
-    r.single = ((one && tt.term_odd[r.start] == tt.term_even[r.start]) ? 1u : 0u) |
-               ((one && tt.term_low[r.start] == 0u) ? 2u : 0u);
+    r.cf = (T)c[0];
+    for (int q = 0; q < 3; ++q) {
+      r.co[q] = (T)c[1 + q];
+      r.ce[q] = (T)c[4 + q];
+    }
     pat[i] = r;
   }
-  for (int i = threadIdx.x; i < nterm; i += blockDim.x) {
-    TermS<T> r;
-    r.co = (T)tt.term_odd[i];
-    r.ce = (T)tt.term_even[i];
-    r.low = tt.term_low[i];
-    term[i] = r;
+  for (int i = threadIdx.x; i < tt.n_grp; i += blockDim.x) {
+    GrpS<T> r;
+    const double* c = tt.grp_coef + (size_t)i * 7;
+    r.low = tt.grp_low[i];
+    r.off = r.low * BS;
+    r.flags = tt.grp_flags[i];
+    r.cf = (T)c[0];
+    for (int q = 0; q < 3; ++q) {
+      r.co[q] = (T)c[1 + q];
+      r.ce[q] = (T)c[4 + q];
+    }
+    grp[i] = r;
   }
+  for (int i = threadIdx.x; i < nlane; i += blockDim.x) {
+    LaneS<T> r;
+    r.co = (T)tt.lane_coef[2 * i];
+    r.ce = (T)tt.lane_coef[2 * i + 1];
+    r.low = tt.lane_low[i];
+    r.off = r.low * BS;
+    lanet[i] = r;
+  }
+  for (int i = threadIdx.x; i < 16; i += blockDim.x) s_reg[i] = (T)tt.reg_coef[i];
   for (int i = threadIdx.x; i < kTileRows; i += blockDim.x) s_low[i] = (T)tt.dg.low[i];
   if (threadIdx.x == 0) {
     for (int i = 0; i < kStages; ++i) {
@@ -918,17 +785,18 @@ __global__ void __launch_bounds__(kTiledThreads, 1) k_spmm_tiled(Layout L, SpmmA
   const int64_t n_tiles = (int64_t)L.n_slices << tile_log;
   const uint32_t tile_mask = (uint32_t)(((int64_t)1 << tile_log) - 1);
   const bool has_prev = a.w_prev != nullptr;
-  // every partner pattern is needed by every tile: the stage sequence is fixed
-  const bool all_active = tt.all_active != 0;
-  const bool partners_flat = tt.partners_flat != 0;
-  const int n_reg0 = tt.n_reg0;
+  // Tiles of a block come in runs of 2^run_log consecutive (slice, tile) places.
+  const int run_log = a.run_log;
+  const int64_t n_runs = n_tiles >> run_log;
+  const int run_mask = (1 << run_log) - 1;
 
   if (warp >= kConsumerWarps) {
-    // ------------------------------------------------ producers (lane 0 of each)
-    // Both walk the whole stage sequence; producer q issues the stages with
-    // seq % kProducerWarps == q (the ring depth is a multiple of kProducerWarps, so
-    // each owns fixed slots).
-    if ((threadIdx.x & 31) != 0) return;
+    // ------------------------------------------------ producers
+    // Both warps walk the whole stage sequence; producer q's lane 0 issues the stages with
+    // seq % kProducerWarps == q (the ring depth is a multiple of kProducerWarps, so each
+    // owns fixed slots). Per tile, ballots over the patterns give the stages it needs: pairs
+    // of patterns consumed together, single-spin patterns, then the others in use.
+    const int pl = threadIdx.x & 31;
     const uint32_t q = (uint32_t)(warp - kConsumerWarps);
     // W_j tiles are reused as partners of neighbouring tiles: keep them in L2;
     // W_{j-1} tiles are read once: let them leave first.
@@ -936,69 +804,93 @@ __global__ void __launch_bounds__(kTiledThreads, 1) k_spmm_tiled(Layout L, SpmmA
     const uint64_t stream = policy_evict_first();
     const uint32_t hk_bytes = (uint32_t)hstride * (uint32_t)sizeof(T);
     const T* const hk_table = reinterpret_cast<const T*>(a.tile_k);
+    const int flat0 = npair + nsingle, nflat = npart - flat0;
     // stage counter kept as (slot, round) so no division by the runtime ring depth
     uint32_t seq = 0, round = 0;
     int slot = 0;
     bool stop = false;
-    for (int64_t gt = blockIdx.x; gt < n_tiles && !stop; gt += gridDim.x) {
-      const int slice = (int)(gt >> tile_log);
-      const uint32_t ut = tt.tile_order[(uint32_t)gt & tile_mask];
-      const size_t soff = (size_t)slice * L.D * BS;
-      const T* W = reinterpret_cast<const T*>(a.w) + soff;
-      const T* Wp = has_prev ? reinterpret_cast<const T*>(a.w_prev) + soff : nullptr;
-      uint32_t zm = 0u, om = 0u;  // pairable groups with their high spin down / up here
-      for (int i = 0; i < npair; ++i) {
-        if (ut & pat[1 + i].high) om |= 1u << i;
-        else zm |= 1u << i;
-      }
-      // stage kinds: -1 = own, -2 = W_{j-1}, p >= 1 = partner pattern p
-      int kind = -1;
-      int pi = 0;  // pairable stages issued
-      while (true) {
-        if (seq % kProducerWarps == q) {
-          if (round > 0 && !ring_wait(&empty[slot], (round - 1u) & 1u, abort_flag)) {
-            stop = true;
-            break;
+    // Waits for the next slot if it is this producer's, has lane 0 call fill(slot address)
+    // and moves on; false when a wait gave up.
+    auto next_stage = [&](uint32_t ut, int what, T c, const void* src, uint32_t extra, const void* src2, uint64_t policy) {
+      if (seq % kProducerWarps == q) {
+        bool ok = true;
+        if (pl == 0) {
+          ok = round == 0 || ring_wait(&empty[slot], (round - 1u) & 1u, abort_flag);
+          if (ok) {
+            unsigned char* dst = ring + (size_t)slot * kSlotBytes;
+            stage[slot].what = what;
+            stage[slot].tile = ut;
+            stage[slot].c = c;
+            fence_proxy_async();
+            mbar_expect_tx(&full[slot], kTileBytes + extra);
+            bulk_load_hint(dst, src, kTileBytes, &full[slot], policy);
+            if (extra) bulk_load_hint(dst + kTileBytes, src2, extra, &full[slot], policy);
           }
-          unsigned char* dst = ring + (size_t)slot * kSlotBytes;
-          fence_proxy_async();
-          if (kind == -1) {
-            mbar_expect_tx(&full[slot], kTileBytes + hk_bytes);
-            bulk_load_hint(dst, W + ((size_t)ut << kTileBits) * BS, kTileBytes, &full[slot], keep);
-            bulk_load_hint(dst + kTileBytes, hk_table + (size_t)ut * hstride, hk_bytes, &full[slot], keep);
-          } else if (kind == -2) {
-            mbar_expect_tx(&full[slot], kTileBytes);
-            bulk_load_hint(dst, Wp + ((size_t)ut << kTileBits) * BS, kTileBytes, &full[slot], stream);
+        }
+        if (!__shfl_sync(0xffffffffu, (int)ok, 0)) stop = true;
+      }
+      ++seq;
+      if (++slot == kStages) {
+        slot = 0;
+        ++round;
+      }
+    };
+    for (int64_t run = blockIdx.x; run < n_runs && !stop; run += gridDim.x)
+      for (int rt = 0; rt <= run_mask && !stop; ++rt) {
+        const int64_t gt = (run << run_log) + rt;
+        const int slice = (int)(gt >> tile_log);
+        const uint32_t ut = tt.tile_order[(uint32_t)gt & tile_mask];
+        const size_t soff = (size_t)slice * L.D * BS;
+        const T* W = reinterpret_cast<const T*>(a.w) + soff;
+        auto tile_of = [&](uint32_t t) { return W + ((size_t)t << kTileBits) * BS; };
+        // pairable groups with their high spin up / down in this tile
+        const bool in_pair = pl < npair;
+        const bool up = in_pair && (ut & pat[pl].high) != 0u;
+        uint32_t om = __ballot_sync(0xffffffffu, up), zm = __ballot_sync(0xffffffffu, in_pair && !up);
+        int n_st = npair + nsingle;
+        for (int f0 = 0; f0 < nflat; f0 += 32) {
+          bool on = false;
+          if (f0 + pl < nflat) {
+            const PatS<T>& A = pat[flat0 + f0 + pl];
+            on = in_use((__popc(ut & A.high) & 1) ? A.co[0] : A.ce[0]);
+          }
+          n_st += __popc(__ballot_sync(0xffffffffu, on));
+        }
+        next_stage(ut, n_st, (T)0, tile_of(ut), hk_bytes, hk_table + (size_t)ut * hstride, keep);
+        for (int joint = __popc(zm) < __popc(om) ? __popc(zm) : __popc(om); (zm | om) && !stop; --joint) {
+          // down and up groups alternate, then the rest of the longer list
+          if (joint > 0) {
+            const int z = __ffs((int)zm) - 1, o = __ffs((int)om) - 1;
+            zm &= zm - 1u;
+            om &= om - 1u;
+            next_stage(ut, z | kJoint, (T)0, tile_of(ut ^ pat[z].high), 0u, nullptr, keep);
+            if (!stop) next_stage(ut, o, (T)0, tile_of(ut ^ pat[o].high), 0u, nullptr, keep);
           } else {
-            mbar_expect_tx(&full[slot], kTileBytes);
-            bulk_load_hint(dst, W + ((size_t)(ut ^ pat[kind].high) << kTileBits) * BS, kTileBytes,
-                           &full[slot], keep);
+            const int p = __ffs((int)(zm | om)) - 1;
+            zm &= ~(1u << p);
+            om &= ~(1u << p);
+            next_stage(ut, p, (T)0, tile_of(ut ^ pat[p].high), 0u, nullptr, keep);
           }
         }
-        ++seq;
-        if (++slot == kStages) {
-          slot = 0;
-          ++round;
+        for (int p = npair; p < flat0 && !stop; ++p)
+          next_stage(ut, p, (T)0, tile_of(ut ^ pat[p].high), 0u, nullptr, keep);
+        for (int f0 = 0; f0 < nflat && !stop; f0 += 32) {
+          T c = (T)0;
+          if (f0 + pl < nflat) {
+            const PatS<T>& A = pat[flat0 + f0 + pl];
+            c = (__popc(ut & A.high) & 1) ? A.co[0] : A.ce[0];
+          }
+          for (uint32_t m = __ballot_sync(0xffffffffu, in_use(c)); m && !stop; m &= m - 1u) {
+            const int i = __ffs((int)m) - 1, p = flat0 + f0 + i;
+            next_stage(ut, p, __shfl_sync(0xffffffffu, c, i), tile_of(ut ^ pat[p].high), 0u, nullptr, keep);
+          }
         }
-        // next stage of this tile
-        if (kind == -2) break;
-        int p;
-        if (pi < npair) {
-          p = pair_pattern(pi++, zm, om);
-        } else {
-          const int from = kind <= npair ? npair + 1 : kind + 1;
-          p = all_active ? from : tiled_next(from, npat, ut, pat);
-        }
-        if (p < npat) {
-          kind = p;
-        } else if (has_prev) {
-          kind = -2;
-        } else {
-          break;
+        if (has_prev && !stop) {
+          const T* Wp = reinterpret_cast<const T*>(a.w_prev) + soff;
+          next_stage(ut, 0, (T)0, Wp + ((size_t)ut << kTileBits) * BS, 0u, nullptr, stream);
         }
       }
-    }
-    if (stop) atomicOr(a.err, 1u);
+    if (stop && pl == 0) atomicOr(a.err, 1u);
     return;
   }
 
@@ -1013,7 +905,8 @@ __global__ void __launch_bounds__(kTiledThreads, 1) k_spmm_tiled(Layout L, SpmmA
   uint32_t rphase = 0;
   bool aborted = false;
   // Waits for the ring slot `ahead` (0 or 1) stages past the next unreleased one.
-  auto acquire = [&](const unsigned char*& slot_ptr, int ahead) -> bool {
+  int at = 0;  // the slot last waited for
+  auto acquire = [&](const T*& slot_ptr, int ahead) -> bool {
     int slot = rslot + ahead;
     uint32_t ph = rphase;
     if (slot >= kStages) {
@@ -1021,7 +914,8 @@ __global__ void __launch_bounds__(kTiledThreads, 1) k_spmm_tiled(Layout L, SpmmA
       ph ^= 1u;
     }
     if (!ring_wait(&full[slot], ph, abort_flag)) return false;
-    slot_ptr = ring + (size_t)slot * kSlotBytes;
+    slot_ptr = reinterpret_cast<const T*>(ring + (size_t)slot * kSlotBytes);
+    at = slot;
     return true;
   };
   auto release = [&]() {
@@ -1064,12 +958,23 @@ __global__ void __launch_bounds__(kTiledThreads, 1) k_spmm_tiled(Layout L, SpmmA
   T* __restrict__ Z = nullptr;
   int cur = -1;       // slice of the tiles in progress
   int unwritten = 0;  // slices [unwritten, n_slices) have no partials yet
+  // Parity of this thread's row group under the in-tile lane terms and groups (bit t).
+  uint32_t act_lane = 0u, act_grp = 0u;
+  for (int t = 0; t < tt.n_own; ++t) act_lane |= (uint32_t)(__popc((uint32_t)rg & lanet[t].low) & 1) << t;
+  for (int t = 0; t < tt.n_grp; ++t) act_grp |= (uint32_t)(((uint32_t)rg & grp[t].low) != 0u) << t;
+  const uint32_t reg_flags = tt.reg_flags;
 
   // The consumers walk the same (slice, tile) sequence as the producers. At every
   // change of slice (and at the end) they close the finished slice; every consumer
   // thread passes the same barriers, also after an abort.
-  for (int64_t gt = blockIdx.x;; gt += gridDim.x) {
-    const int slice = gt < n_tiles ? (int)(gt >> tile_log) : L.n_slices;
+  int64_t run = blockIdx.x;
+  for (int rt = 0;; ++rt) {
+    if (rt > run_mask) {
+      rt = 0;
+      run += gridDim.x;
+    }
+    const int64_t gt = (run << run_log) + rt;
+    const int slice = run < n_runs ? (int)(gt >> tile_log) : L.n_slices;
     if (slice != cur) {
       if (consumers_sync_or(aborted)) aborted = true;
       if (MODE == kModePass1 && !aborted) {
@@ -1120,211 +1025,205 @@ __global__ void __launch_bounds__(kTiledThreads, 1) k_spmm_tiled(Layout L, SpmmA
     }
     if (aborted) continue;
 
-    const uint32_t ut = tt.tile_order[(uint32_t)gt & tile_mask];
-    const uint32_t row0 = ut << kTileBits;
-    const unsigned char* sp;
+    // (the tile's index: from the table for the uniform terms, whose tiles are short, else
+    // with the own tile's stage -- 1% and 5% better so)
+    uint32_t ut = UNI ? tt.tile_order[(uint32_t)gt & tile_mask] : 0u;
+    const T* sp;
     // own tile: diagonal and in-tile terms
     if (!acquire(sp, 0)) {
       aborted = true;
       continue;
     }
-    const T* own = reinterpret_cast<const T*>(sp);
+    const T* const own = sp;
+    const int n_st = stage[at].what;
+    if constexpr (!UNI) ut = stage[at].tile;
+    const uint32_t row0 = ut << kTileBits;
     T xo[RPT][VW], y[RPT][VW];
     {
       T dg[RPT];
-      tile_diagonal<T, RPT, RG>(dg, s_low, reinterpret_cast<const T*>(sp + kTileBytes), rg, tt.dg);
+      tile_diagonal<T, RPT, RG>(dg, s_low, own + kTileBytes / sizeof(T), rg, tt.dg);
+      load_rows<kStep>(xo, own + rgoff);
 #pragma unroll
-      for (int m = 0; m < RPT; ++m) {
-        VecIO<T, VW>::ld_rw(xo[m], own + rgoff + m * kStep);
+      for (int m = 0; m < RPT; ++m)
 #pragma unroll
         for (int v = 0; v < VW; ++v) y[m][v] = dg[m] * xo[m][v];
-      }
     }
-    const int t1 = pat[0].end, tr = pat[0].start + n_reg0;
-    for (int t = pat[0].start; t < tr; ++t) {  // masks on the register rows only
-      const TermS<T> d = term[t];
-      switch (d.low >> RGL) {
-        case 1: reg_flip<1, RG, UNI>(y, xo, rg, d.low, d.co, d.ce); break;
-        case 2: reg_flip<2, RG, UNI>(y, xo, rg, d.low, d.co, d.ce); break;
-        case 3: reg_flip<3, RG, UNI>(y, xo, rg, d.low, d.co, d.ce); break;
-        case 4: reg_flip<4, RG, UNI>(y, xo, rg, d.low, d.co, d.ce); break;
-        case 5: reg_flip<5, RG, UNI>(y, xo, rg, d.low, d.co, d.ce); break;
-        case 6: reg_flip<6, RG, UNI>(y, xo, rg, d.low, d.co, d.ce); break;
-        default: reg_flip<7, RG, UNI>(y, xo, rg, d.low, d.co, d.ce); break;
-      }
+    // fields and hops of the register rows alone
+    if (reg_flags & 2u) reg_uniform<1>(y, xo, s_reg[8 + 1], s_reg[1]);
+    if (reg_flags & 4u) reg_uniform<2>(y, xo, s_reg[8 + 2], s_reg[2]);
+    if (reg_flags & 16u) reg_uniform<4>(y, xo, s_reg[8 + 4], s_reg[4]);
+    if constexpr (!UNI) {
+      if (reg_flags & 8u) reg_uniform<3>(y, xo, s_reg[8 + 3], s_reg[3]);
+      if (reg_flags & 32u) reg_uniform<5>(y, xo, s_reg[8 + 5], s_reg[5]);
+      if (reg_flags & 64u) reg_uniform<6>(y, xo, s_reg[8 + 6], s_reg[6]);
+    } else if (reg_flags & (8u | 32u | 64u)) {
+      reg_uniform<3>(y, xo, s_reg[8 + 3], s_reg[3]);
+      reg_uniform<5>(y, xo, s_reg[8 + 5], s_reg[5]);
+      reg_uniform<6>(y, xo, s_reg[8 + 6], s_reg[6]);
     }
-    for (int t = tr; t < t1;) {
-      const TermS<T> d = term[t];
-      if (d.co == d.ce && t + 1 < t1) {
-        const TermS<T> d2 = term[t + 1];
-        if (d2.co == d2.ce) {
-          apply2_uniform<T, VW, RPT, RG, BS>(y, rgoff, own, d.low, d.co, own, d2.low, d2.co);
-          t += 2;
-          continue;
-        }
+    // a row-group spin's field and its hops with the register spins share one set of loads
+    for (int t = 0; t < tt.n_grp; ++t) {
+      const GrpS<T>& G = grp[t];
+      const bool odd = (act_grp >> t) & 1u;
+      const uint32_t fl = G.flags;
+      T xp[RPT][VW];
+      load_rows<kStep>(xp, own + (rgoff ^ (int)G.off));
+      if (fl & kPatField) {
+        const T c = G.cf;
+#pragma unroll
+        for (int m = 0; m < RPT; ++m) axpy(y[m], c, xp[m]);
       }
-      apply_term<T, VW, RPT, RG, BS, UNI>(y, rgoff, rg, own, d.low, d.low, d.co, d.ce, 0u);
-      ++t;
+      if (fl & kPatReg) reg_lanes<1>(y, xp, odd ? G.co[0] : G.ce[0], odd ? G.ce[0] : G.co[0]);
+      if (fl & (kPatReg << 1)) reg_lanes<2>(y, xp, odd ? G.co[1] : G.ce[1], odd ? G.ce[1] : G.co[1]);
+      if (fl & (kPatReg << 2)) reg_lanes<4>(y, xp, odd ? G.co[2] : G.ce[2], odd ? G.ce[2] : G.co[2]);
+    }
+    // terms of the row-group spins alone
+    if constexpr (UNI) {
+      int t = 0;
+      for (; t + 1 < tt.n_own; t += 2)
+        rows_fma2<kStep>(y, own + (rgoff ^ (int)lanet[t].off), lanet[t].co, own + (rgoff ^ (int)lanet[t + 1].off),
+                         lanet[t + 1].co);
+      if (t < tt.n_own) rows_fma<kStep>(y, own + (rgoff ^ (int)lanet[t].off), lanet[t].co);
+    } else {
+      for (int t = 0; t < tt.n_own; ++t) {
+        const LaneS<T> d = lanet[t];
+        const T c = ((act_lane >> t) & 1u) ? d.co : d.ce;
+        // where the coefficient differs across the warp's lanes they all run the term
+        if (__any_sync(0xffffffffu, in_use(c))) rows_fma<kStep>(y, own + (rgoff ^ (int)d.off), c);
+      }
     }
     release();
-    // the terms of one partner pattern A, copied to P (any coefficients)
-    auto pattern_terms = [&](const PatS<T>& A, const T* P) {
-      const uint32_t hi_bits = A.high << kTileBits;
-      for (int t = A.start; t < A.end;) {
-        const TermS<T> d = term[t];
-        if (d.co == d.ce && t + 1 < A.end) {
-          const TermS<T> d2 = term[t + 1];
-          if (d2.co == d2.ce) {
-            apply2_uniform<T, VW, RPT, RG, BS>(y, rgoff, P, d.low, d.co, P, d2.low, d2.co);
-            t += 2;
-            continue;
-          }
+    // Partner tiles, in the producer's order: opposite-spin pairs, single-spin patterns, the
+    // flat ones in use.
+    auto single = [&](const PatS<T>& A) {  // one high spin: its field and its hops
+      const uint32_t hs = (ut & A.high) != 0u, fl = A.flags;
+      if (fl & (kPatField | (kPatReg * 7u))) {
+        T xp[RPT][VW];
+        load_rows<kStep>(xp, sp + rgoff);
+        if (fl & kPatField) {
+          const T c = A.cf;
+#pragma unroll
+          for (int m = 0; m < RPT; ++m) axpy(y[m], c, xp[m]);
         }
-        apply_term<T, VW, RPT, RG, BS, UNI>(y, rgoff, rg, P, d.low, d.low | hi_bits, d.co, d.ce, row0);
-        ++t;
+        if (fl & kPatReg) reg_uniform<1>(y, xp, hs ? A.co[0] : A.ce[0], hs ? A.ce[0] : A.co[0]);
+        if (fl & (kPatReg << 1)) reg_uniform<2>(y, xp, hs ? A.co[1] : A.ce[1], hs ? A.ce[1] : A.co[1]);
+        if (fl & (kPatReg << 2)) reg_uniform<4>(y, xp, hs ? A.co[2] : A.ce[2], hs ? A.ce[2] : A.co[2]);
+      }
+      for (int t = A.start; t < A.end; ++t) {
+        const LaneS<T> d = lanet[t];
+        const bool odd = (((uint32_t)rg & d.low) != 0u) != (hs != 0u);
+        const T c = UNI || odd ? d.co : d.ce;
+        if (UNI || __any_sync(0xffffffffu, in_use(c))) rows_fma<kStep>(y, sp + (rgoff ^ (int)d.off), c);
       }
     };
-    if constexpr (!UNI) {
-      // pairable partner tiles: a group with its high spin down and one with it up
-      // together, then the rest of the longer list one by one
-      if (npair > 0) {
-        uint32_t zm = 0u, om = 0u;
-        for (int q = 0; q < npair; ++q) {
-          if (ut & pat[1 + q].high) om |= 1u << q;
-          else zm |= 1u << q;
-        }
-        const int nz = __popc(zm), no = __popc(om);
-        const int n2 = 2 * (nz < no ? nz : no);
-        for (int i = 0; i < npair;) {
-          const PatS<T> A = pat[pair_pattern(i, zm, om)];
-          if (i < n2) {
-            const PatS<T> B = pat[pair_pattern(i + 1, zm, om)];
-            const unsigned char* sp2;
-            if (!acquire(sp, 0) || !acquire(sp2, 1)) {
-              aborted = true;
-              break;
-            }
-            apply_paired<T, VW, RPT, RG, BS>(y, rgoff, rg, reinterpret_cast<const T*>(sp),
-                                             reinterpret_cast<const T*>(sp2), term + A.start, term + B.start,
-                                             A.end - A.start);
-            release2();
-            i += 2;
-          } else {
-            if (!acquire(sp, 0)) {
-              aborted = true;
-              break;
-            }
-            pattern_terms(A, reinterpret_cast<const T*>(sp));
-            release();
-            ++i;
-          }
-        }
-        if (aborted) continue;
-      }
-    }
-    // partner tiles; two single-term patterns are consumed together so their
-    // shared-memory loads overlap
-    if (partners_flat) {
-      // one uniform term per partner tile, partner row = same row: no term records
-      int p = 1;
-      for (; p + 1 < npat; p += 2) {
-        const T cA = pat[p].c0, cB = pat[p + 1].c0;
-        const unsigned char* sb;
-        if (!acquire(sp, 0) || !acquire(sb, 1)) {
+    if constexpr (UNI) {
+      for (int st = 0; st < n_st;) {
+        if (!acquire(sp, 0)) {
           aborted = true;
           break;
         }
-        const T* PA = reinterpret_cast<const T*>(sp) + rgoff;
-        const T* PB = reinterpret_cast<const T*>(sb) + rgoff;
-#pragma unroll
-        for (int m = 0; m < RPT; ++m) {
-          T u[VW], w[VW];
-          VecIO<T, VW>::ld_rw(u, PA + m * kStep);
-          VecIO<T, VW>::ld_rw(w, PB + m * kStep);
-#pragma unroll
-          for (int v = 0; v < VW; ++v) y[m][v] = fma(cB, w[v], fma(cA, u[v], y[m][v]));
+        const int p = stage[at].what;
+        if (p < nsingle) {
+          single(pat[p]);
+          release();
+          ++st;
+          continue;
+        }
+        const T cA = stage[at].c;
+        if (n_st - st > 1) {  // two at a time: their loads overlap
+          const T* sb;
+          if (!acquire(sb, 1)) {
+            aborted = true;
+            break;
+          }
+          rows_fma2<kStep>(y, sp + rgoff, cA, sb + rgoff, stage[at].c);
+          release2();
+          st += 2;
+        } else {
+          rows_fma<kStep>(y, sp + rgoff, cA);
+          release();
+          ++st;
+        }
+      }
+    } else {
+      for (int st = 0; st < npair;) {
+        if (!acquire(sp, 0)) {
+          aborted = true;
+          break;
+        }
+        const int what = stage[at].what;
+        const PatS<T>& A = pat[what & (kJoint - 1)];
+        if (!(what & kJoint)) {
+          single(A);
+          release();
+          ++st;
+          continue;
+        }
+        // A group whose high spin is down (here) and one whose is up (the next stage), with the
+        // same in-tile partners: term l of the first acts on the rows whose spin l is up, of the
+        // second on the others, so every row takes exactly one of the two.
+        const T* sb;
+        if (!acquire(sb, 1)) {
+          aborted = true;
+          break;
+        }
+        const PatS<T>& B = pat[stage[at].what];
+        const uint32_t fl = A.flags;
+        if (fl & (kPatReg * 7u)) {
+          T xp[RPT][VW];
+          load_rows<kStep>(xp, sp + rgoff);
+          if (fl & kPatReg) reg_half<1, 1>(y, xp, A.co[0]);
+          if (fl & (kPatReg << 1)) reg_half<2, 1>(y, xp, A.co[1]);
+          if (fl & (kPatReg << 2)) reg_half<4, 1>(y, xp, A.co[2]);
+          load_rows<kStep>(xp, sb + rgoff);
+          if (fl & kPatReg) reg_half<1, 0>(y, xp, B.co[0]);
+          if (fl & (kPatReg << 1)) reg_half<2, 0>(y, xp, B.co[1]);
+          if (fl & (kPatReg << 2)) reg_half<4, 0>(y, xp, B.co[2]);
+        }
+        const int n = A.end - A.start;
+        const LaneS<T>* const la = lanet + A.start;
+        const LaneS<T>* const lb = lanet + B.start;
+        for (int t = 0; t < n; ++t) {
+          const bool up = ((uint32_t)rg & la[t].low) != 0u;
+          rows_fma<kStep>(y, (up ? sp : sb) + (rgoff ^ (int)la[t].off), up ? la[t].co : lb[t].co);
         }
         release2();
+        st += 2;
       }
-      if (!aborted && p < npat) {
-        const T cA = pat[p].c0;
+      if (aborted) continue;
+      for (int p = npair; p < npair + nsingle; ++p) {
+        if (!acquire(sp, 0)) {
+          aborted = true;
+          break;
+        }
+        single(pat[p]);
+        release();
+      }
+      if (aborted) continue;
+      // partner rows are the same rows: one coefficient per tile, from the producer
+      int left = n_st - npair - nsingle;
+      for (; left > 1; left -= 2) {
+        const T* sb;
+        if (!acquire(sp, 0)) {
+          aborted = true;
+          break;
+        }
+        const T cA = stage[at].c;
+        if (!acquire(sb, 1)) {
+          aborted = true;
+          break;
+        }
+        rows_fma2<kStep>(y, sp + rgoff, cA, sb + rgoff, stage[at].c);
+        release2();
+      }
+      if (!aborted && left) {
         if (!acquire(sp, 0)) {
           aborted = true;
         } else {
-          const T* PA = reinterpret_cast<const T*>(sp) + rgoff;
-#pragma unroll
-          for (int m = 0; m < RPT; ++m) {
-            T u[VW];
-            VecIO<T, VW>::ld_rw(u, PA + m * kStep);
-#pragma unroll
-            for (int v = 0; v < VW; ++v) y[m][v] = fma(cA, u[v], y[m][v]);
-          }
+          rows_fma<kStep>(y, sp + rgoff, stage[at].c);
           release();
         }
       }
-    } else
-    for (int p = all_active ? npair + 1 : tiled_next(npair + 1, npat, ut, pat); p < npat;) {
-      const int pn = all_active ? p + 1 : tiled_next(p + 1, npat, ut, pat);
-      const PatS<T> A = pat[p];
-      if (A.single & 2u) {
-        // One term whose partner row is the same row (m_low = 0): its coefficient is
-        // the same for every row of this tile (the parity of its mask is that of the
-        // tile bits). Two such partner tiles are consumed together when they follow
-        // each other.
-        const T cA = (__popc(ut & A.high) & 1) ? A.c0 : A.c1;
-        if (pn < npat && (pat[pn].single & 2u)) {
-          const PatS<T> Bq = pat[pn];
-          const T cB = (__popc(ut & Bq.high) & 1) ? Bq.c0 : Bq.c1;
-          const unsigned char* sp2;
-          if (!acquire(sp, 0) || !acquire(sp2, 1)) {
-            aborted = true;
-            break;
-          }
-          apply2_uniform<T, VW, RPT, RG, BS>(y, rgoff, reinterpret_cast<const T*>(sp), 0u, cA,
-                                             reinterpret_cast<const T*>(sp2), 0u, cB);
-          release2();
-          p = all_active ? pn + 1 : tiled_next(pn + 1, npat, ut, pat);
-          continue;
-        }
-        if (!acquire(sp, 0)) {
-          aborted = true;
-          break;
-        }
-        const T* PA = reinterpret_cast<const T*>(sp) + rgoff;
-#pragma unroll
-        for (int m = 0; m < RPT; ++m) {
-          T u[VW];
-          VecIO<T, VW>::ld_rw(u, PA + m * kStep);
-#pragma unroll
-          for (int v = 0; v < VW; ++v) y[m][v] = fma(cA, u[v], y[m][v]);
-        }
-        release();
-        p = pn;
-        continue;
-      }
-      if (pn < npat && A.single) {
-        const PatS<T> Bq = pat[pn];
-        if (Bq.single) {
-          const unsigned char* sp2;
-          if (!acquire(sp, 0) || !acquire(sp2, 1)) {
-            aborted = true;
-            break;
-          }
-          apply2_uniform<T, VW, RPT, RG, BS>(y, rgoff, reinterpret_cast<const T*>(sp), A.low0, A.c0,
-                                             reinterpret_cast<const T*>(sp2), Bq.low0, Bq.c0);
-          release();
-          release();
-          p = all_active ? pn + 1 : tiled_next(pn + 1, npat, ut, pat);
-          continue;
-        }
-      }
-      if (!acquire(sp, 0)) {
-        aborted = true;
-        break;
-      }
-      pattern_terms(A, reinterpret_cast<const T*>(sp));
-      release();
-      p = pn;
     }
     if (aborted) continue;
     // Z = (H W) M + W_prev Cp, row by row, with the W_j^T Z partial sums
@@ -1334,7 +1233,7 @@ __global__ void __launch_bounds__(kTiledThreads, 1) k_spmm_tiled(Layout L, SpmmA
         aborted = true;
         continue;
       }
-      Pp = reinterpret_cast<const T*>(sp);
+      Pp = sp;
     }
     T* const zrow = Z + (size_t)row0 * BS + rgoff;  // this thread's first row of the tile
     if constexpr (MODE == kModeApply) {  // Z = H W
@@ -2489,6 +2388,27 @@ cudaError_t launch_tile_diag(const Layout& L, const TileDiag& dg, void* out, cud
   return cudaGetLastError();
 }
 
+// Runs of 2^r consecutive tiles per block: a block closes its partial sums and loads the
+// mixing coefficients at every change of slice, which costs about a third of a tile's time,
+// so slices of few tiles (N = 16: 64 tiles, fewer than the 152 blocks) are walked in runs.
+// The r with the smallest largest block, counting that; 0 for slices of many tiles.
+static int tiled_run_log(const Layout& L) {
+  const int64_t per = L.D >> kTileBits, total = per * L.n_slices, grid = spmm_tiled_grid(L);
+  int best = 0;
+  double least = 1e300;
+  for (int r = 0; r <= 3 && (1 << r) <= per; ++r) {
+    const int64_t runs = total >> r, mine = (runs + grid - 1) / grid;
+    // slices a block enters: one per run, or per pass over a slice longer than the stride
+    const double slices = std::min<double>((double)mine, (double)(mine * grid << r) / (double)per + 1.0);
+    const double cost = (double)(mine << r) + 0.35 * slices;
+    if (cost < 0.999 * least) {
+      least = cost;
+      best = r;
+    }
+  }
+  return best;
+}
+
 template <typename T, int DS, int MODE, bool UNI = false>
 static cudaError_t launch_tiled(const Layout& L, const SpmmArgs& a0, cudaStream_t st) {
   cudaError_t e = opt_in_smem(reinterpret_cast<const void*>(k_spmm_tiled<T, DS, MODE, UNI>));
@@ -2505,37 +2425,36 @@ static cudaError_t launch_tiled(const Layout& L, const SpmmArgs& a0, cudaStream_
   const TiledTerms& tt = a.tiled;
   a.stages = 6;  // a multiple of kProducerWarps
   while (a.stages > kProducerWarps &&
-         tiled_smem_bytes<T>(tt.n_pat, tt.n_terms, tt.dg.n_entries, a.stages) > (size_t)optin)
+         tiled_smem_bytes<T>(tt.n_part, tt.n_lane, tt.n_grp, tt.dg.n_entries, a.stages) > (size_t)optin)
     a.stages -= kProducerWarps;
-  const size_t sm = tiled_smem_bytes<T>(tt.n_pat, tt.n_terms, tt.dg.n_entries, a.stages);
+  a.run_log = tiled_run_log(L);
+  const size_t sm = tiled_smem_bytes<T>(tt.n_part, tt.n_lane, tt.n_grp, tt.dg.n_entries, a.stages);
   if (sm > (size_t)optin) return cudaErrorInvalidValue;
   k_spmm_tiled<T, DS, MODE, UNI><<<dim3((unsigned)spmm_tiled_grid(L), 1), kTiledThreads, sm, st>>>(L, a);
   return cudaGetLastError();
 }
 
 cudaError_t launch_spmm(const Layout& L, int mode, const SpmmArgs& a, cudaStream_t st) {
-  if (layout_tiled(L) && a.tiled.n_pat > 0 && a.tile_k) {
+  if (layout_tiled(L) && a.tiled.ready && a.tile_k) {
     const bool f32 = L.precision == RDM_FP32;
     if (mode == kModeApply) {
       if (L.DS != 1) return cudaErrorInvalidValue;
       return f32 ? launch_tiled<float, 1, kModeApply>(L, a, st) : launch_tiled<double, 1, kModeApply>(L, a, st);
     }
-    const bool p1 = mode == kModePass1;
-    if (f32 && a.tiled.all_uniform) {  // no parity-dependent coefficient anywhere
-      if (L.DS == 1)
-        return p1 ? launch_tiled<float, 1, kModePass1, true>(L, a, st) : launch_tiled<float, 1, kModePass2, true>(L, a, st);
-      if (L.DS == 2)
-        return p1 ? launch_tiled<float, 2, kModePass1, true>(L, a, st) : launch_tiled<float, 2, kModePass2, true>(L, a, st);
-      return p1 ? launch_tiled<float, 4, kModePass1, true>(L, a, st) : launch_tiled<float, 4, kModePass2, true>(L, a, st);
-    }
-    if (f32) {
-      if (L.DS == 1) return p1 ? launch_tiled<float, 1, kModePass1>(L, a, st) : launch_tiled<float, 1, kModePass2>(L, a, st);
-      if (L.DS == 2) return p1 ? launch_tiled<float, 2, kModePass1>(L, a, st) : launch_tiled<float, 2, kModePass2>(L, a, st);
-      return p1 ? launch_tiled<float, 4, kModePass1>(L, a, st) : launch_tiled<float, 4, kModePass2>(L, a, st);
-    }
-    if (L.DS == 1) return p1 ? launch_tiled<double, 1, kModePass1>(L, a, st) : launch_tiled<double, 1, kModePass2>(L, a, st);
-    if (L.DS == 2) return p1 ? launch_tiled<double, 2, kModePass1>(L, a, st) : launch_tiled<double, 2, kModePass2>(L, a, st);
-    return p1 ? launch_tiled<double, 4, kModePass1>(L, a, st) : launch_tiled<double, 4, kModePass2>(L, a, st);
+    // UNI: no parity-dependent coefficient anywhere
+    const bool uni = a.tiled.all_uniform != 0, p1 = mode == kModePass1;
+    auto go = [&](auto t, auto ds) -> cudaError_t {
+      using T = decltype(t);
+      constexpr int DS = decltype(ds)::value;
+      if (uni) return p1 ? launch_tiled<T, DS, kModePass1, true>(L, a, st) : launch_tiled<T, DS, kModePass2, true>(L, a, st);
+      return p1 ? launch_tiled<T, DS, kModePass1>(L, a, st) : launch_tiled<T, DS, kModePass2>(L, a, st);
+    };
+    auto by_ds = [&](auto t) -> cudaError_t {
+      if (L.DS == 1) return go(t, std::integral_constant<int, 1>{});
+      if (L.DS == 2) return go(t, std::integral_constant<int, 2>{});
+      return go(t, std::integral_constant<int, 4>{});
+    };
+    return f32 ? by_ds(float{}) : by_ds(double{});
   }
   RDM_DISPATCH(L, {
     const size_t sm = terms_smem<T>(a.n_flip, a.n_diag);

@@ -154,11 +154,13 @@ rdm_status estimate_impl(rdm_ham* ham, cudaStream_t s, char* ws, size_t ws_bytes
 // the tiled SpMM's pattern tables), uploaded with one copy.
 struct TermImage {
   std::vector<unsigned char> bytes;
-  size_t off_flips = 0, off_diags = 0, off_pat_high = 0, off_pat_start = 0, off_pat_flags = 0,
-         off_term_low = 0, off_term_odd = 0, off_term_even = 0, off_dg_low = 0, off_dg_mlo = 0,
-         off_dg_hstart = 0, off_dg_thi = 0, off_dg_tc = 0, off_dg_slot = 0, off_tile_order = 0;
-  int n_pat = 0, n_pair = 0, n_terms = 0, all_active = 1, partners_flat = 0, all_uniform = 1, n_reg0 = 0, n_dg_groups = 0,
-      n_dg_terms = 0, dg_entries = 0;
+  size_t off_flips = 0, off_diags = 0, off_pat_high = 0, off_pat_start = 0, off_pat_flags = 0, off_pat_coef = 0,
+         off_lane_low = 0, off_lane_coef = 0, off_grp_low = 0, off_grp_flags = 0, off_grp_coef = 0, off_reg_coef = 0,
+         off_dg_low = 0, off_dg_mlo = 0, off_dg_hstart = 0, off_dg_thi = 0, off_dg_tc = 0, off_dg_slot = 0,
+         off_tile_order = 0;
+  int tiled = 0, n_part = 0, n_pair = 0, n_single = 0, n_lane = 0, n_own = 0, n_grp = 0, all_uniform = 1,
+      n_dg_groups = 0, n_dg_terms = 0, dg_entries = 0;
+  uint32_t reg_flags = 0;
   uint32_t dg_dep = 0;
   int dg_off[8] = {};
 };

@@ -113,9 +113,7 @@ cudaError_t launch_gauss_fill(const Layout& L, int n_v, uint64_t seed, int64_t l
 // states into each byte of L2, so the partner tiles of a tile stay cached. A flip
 // mask m splits into m_high = m >> kTileBits (which tile the partner row lies in,
 // relative to this one: tile ^ m_high) and m_low (the row permutation inside that
-// tile). Pattern p collects the terms with one m_high; pattern 0 has m_high = 0
-// (in-tile terms). Flags: bit0 = every term has m_low = 0 (its activity is uniform
-// over a tile), bit1/bit2 = some c_odd/c_even is nonzero.
+// tile). Each distinct nonzero m_high is a partner pattern: one tile copy (TiledTerms).
 constexpr int kTiledLanesLog = 1;
 constexpr int kTiledLanes = 1 << kTiledLanesLog;
 constexpr int kTileBits = 11 - kTiledLanesLog;
@@ -161,21 +159,33 @@ RDM_HD inline int tile_diag_stride(int n_entries, int elem) {
   return (n_entries + per16 - 1) / per16 * per16;
 }
 
+// The flip terms by where their one or two flipped spins sit: above the tile (high), in a
+// consumer thread's register rows (the top kTileRegBits tile bits) or in the row group (the
+// bits below). Partner patterns (one per distinct m_high) come in three kinds, in this order:
+//   pairs   one high spin whose hops with in-tile spins are parity-only (c_even = 0) and have
+//           the same partners in every such pattern (consumed in opposite-spin pairs);
+//   single  one high spin with any in-tile hops;
+//   flat    the partner row is the same row: two high spins, or a field on one high spin. The
+//           coefficient (co[0] / ce[0] by the parity of the tile's bits) is one per tile.
+constexpr uint32_t kPatField = 1u;  // the high (or group) spin has a field: cf
+constexpr uint32_t kPatReg = 2u;    // << a: a hop with register spin a: co[a], ce[a]
 struct TiledTerms {
-  int n_pat;
-  int n_pair;                 // patterns 1..n_pair: one high spin, the same in-tile hop
-                              // partners, parity-only (consumed in opposite-spin pairs)
-  int n_terms;
-  int all_active;             // 1: every tile needs every partner pattern
-  int partners_flat;          // 1: and each is one uniform term with m_low = 0
+  int ready;                  // the tables below are there
+  int n_part, n_pair, n_single;  // partner patterns; the rest after pairs and singles are flat
+  int n_lane, n_own;          // lane terms; the first n_own are in-tile
+  int n_grp;                  // row-group spins with hops to register spins (in-tile)
   int all_uniform;            // 1: every term has c_odd = c_even
-  int n_reg0;                 // leading in-tile terms that act on register rows only
-  const uint32_t* pat_high;   // [n_pat]
-  const int* pat_start;       // [n_pat + 1]
-  const uint32_t* pat_flags;  // [n_pat]
-  const uint32_t* term_low;   // [n_terms]
-  const double* term_odd;     // [n_terms]
-  const double* term_even;    // [n_terms]
+  uint32_t reg_flags;         // bit K: an in-tile term on register mask K (1..7)
+  const uint32_t* pat_high;   // [n_part]
+  const int* pat_start;       // [n_part + 1] lane terms of a pattern
+  const uint32_t* pat_flags;  // [n_part] kPatField, kPatReg
+  const double* pat_coef;     // [n_part][7] cf, co[3], ce[3]
+  const uint32_t* lane_low;   // [n_lane] m_low, row-group bits only
+  const double* lane_coef;    // [n_lane][2] c_odd, c_even
+  const uint32_t* grp_low;    // [n_grp] the row-group spin's bit
+  const uint32_t* grp_flags;  // [n_grp]
+  const double* grp_coef;     // [n_grp][7]
+  const double* reg_coef;     // [16] c_odd[8], c_even[8] by register mask
   const uint32_t* tile_order;  // [tiles per slice]: the walk's k-th tile of a slice
   TileDiag dg;
 };
@@ -196,10 +206,11 @@ struct SpmmArgs {
   const double* e;     // [nb][group][DS*DS]
   int nb;
   int psi_first;       // 1: psi = w E (no read)
-  TiledTerms tiled;    // n_pat = 0: not available
+  TiledTerms tiled;    // ready = 0: not available
   const void* tile_k;  // [tiles][stride] A table of the tiled diagonal (launch_tile_diag)
   uint32_t* err;       // bit 0 set if a bulk-copy wait gave up
   int stages;          // tiled SpMM: copy-ring depth (set by the launcher)
+  int run_log;         // and log2 of the consecutive tiles a block takes at a time
 };
 
 // True if the tiled SpMM applies to this layout: rows of kTiledLanes 16-byte vectors
