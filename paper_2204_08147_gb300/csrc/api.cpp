@@ -2012,7 +2012,8 @@ rdm_status EstimateRun::finish_rest() {
     });
     host_ms += std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - coef_t0).count();
     for (int bi = 0; bi < nb; ++bi) {
-      const int kb = *std::max_element(jlast.begin() + (size_t)bi * n_v, jlast.begin() + (size_t)(bi + 1) * n_v);
+      const int kb =
+          std::max(1, *std::max_element(jlast.begin() + (size_t)bi * n_v, jlast.begin() + (size_t)(bi + 1) * n_v));
       kbeta[bi] = kb;
       for (int j = kb; j < k; ++j) {  // E_j of this beta beyond its last needed step
         double* e0p = &hE[((size_t)j * p.nbc + bi) * (e_view ? ngo * nvo : ng * nv)];
