@@ -1500,10 +1500,19 @@ class EstimateRun {
   double* d_betas = nullptr;
   char* d_jobs = nullptr;
   bool dense_on_device = false;
+  bool coef_on_device = false;  // the Gram coefficients too (nothing of c, M, T comes back)
   double thr_abs_sq = 0, thr_rel_sq = 0;
   SpmmArgs sa{};
   double blk_b = 0;
   uint64_t h2d = 0, d2h = 0;
+  // bytes of f, quad, jlast and kb (device_coefficients), each rounded up to 8
+  size_t coef_scratch() const {
+    return (size_t)n_beta * n_v * (sizeof(double) * (1 + (size_t)nv) + sizeof(int)) + (size_t)n_beta * sizeof(int) + 16;
+  }
+  double gram_tau() const {
+    return 1e-3 * (o->precision == RDM_FP32 ? 1.1920928955078125e-07 : 2.220446049250313e-16);
+  }
+  rdm_status device_coefficients(double e0, std::vector<double>& quad, std::vector<int>& kbeta);
   int cur = 0, prv = -1, nxt = 1;
   std::vector<double> ta, tb, mz, cstore, tmin;
   std::vector<char> okv;
@@ -1772,16 +1781,31 @@ rdm_status EstimateRun::pass1() {
 }
 
 rdm_status EstimateRun::fetch_t() {
-  ta.assign((size_t)k * cstride, 0.0);
-  tb.assign((size_t)k * cstride, 0.0);
-  mz.assign((size_t)(k + 1) * cstride, 0.0);
+  const int mode = ham->ctx ? ham->ctx->device_dense : 1;
+  wants_device = p.dev_dense && (mode == 2 || (mode == 1 && n_beta >= kDeviceDenseMinBetas));
+  // With the basis stored and block recurrences, the coefficients are formed where c is.
+  // On the host they took the copies of c and E (52 MB each way for 64 vectors, 64 betas and
+  // 100 steps of d_s = 4) and about 1 ms per solve of the small batch. Their scratch is the
+  // Chebyshev vectors' (dead once c is formed).
+  coef_on_device = wants_device && store && !p.single && n_beta <= 65535 &&
+                   coef_scratch() <= (size_t)ng * p.vstride * k * nv * sizeof(double);
+  const bool t_back = !wants_device || out->t_a || out->t_b;
   uint32_t flags[4];
-  CK(cudaMemcpyAsync(ta.data(), d_ta, ta.size() * sizeof(double), cudaMemcpyDeviceToHost, s));
-  CK(cudaMemcpyAsync(tb.data(), d_tb, tb.size() * sizeof(double), cudaMemcpyDeviceToHost, s));
-  CK(cudaMemcpyAsync(mz.data(), MZ(1), mz.size() * sizeof(double), cudaMemcpyDeviceToHost, s));
+  d2h += sizeof flags;
+  if (t_back) {
+    ta.assign((size_t)k * cstride, 0.0);
+    tb.assign((size_t)k * cstride, 0.0);
+    CK(cudaMemcpyAsync(ta.data(), d_ta, ta.size() * sizeof(double), cudaMemcpyDeviceToHost, s));
+    CK(cudaMemcpyAsync(tb.data(), d_tb, tb.size() * sizeof(double), cudaMemcpyDeviceToHost, s));
+    d2h += (ta.size() + tb.size()) * sizeof(double);
+  }
+  if (!coef_on_device) {
+    mz.assign((size_t)(k + 1) * cstride, 0.0);
+    CK(cudaMemcpyAsync(mz.data(), MZ(1), mz.size() * sizeof(double), cudaMemcpyDeviceToHost, s));
+    d2h += mz.size() * sizeof(double);
+  }
   CK(cudaMemcpyAsync(flags, d_flags, sizeof flags, cudaMemcpyDeviceToHost, s));
   CK(cudaStreamSynchronize(s));
-  d2h += (ta.size() + tb.size() + mz.size()) * sizeof(double) + sizeof flags;
   if (flags[1]) {
     set_error("a bulk-copy wait in the SpMM kernel gave up (device error)");
     return RDM_ECUDA;
@@ -1794,12 +1818,10 @@ rdm_status EstimateRun::fetch_t() {
   // per-recurrence shift t_min(r); E0 = min_r t_min(r) (Sec. 3.2), then rescaling. A
   // recurrence r is bath vector r (block) or column r = l dso + i (single).
   const int n = k * ds;
-  cstore.assign((size_t)n_rec * n_beta * n * ds, 0.0);
+  if (!coef_on_device) cstore.assign((size_t)n_rec * n_beta * n * ds, 0.0);
   tmin.assign(n_rec, 0.0);
   okv.assign(n_rec, 1);
   dense_on_device = false;
-  const int mode = ham->ctx ? ham->ctx->device_dense : 1;
-  wants_device = p.dev_dense && (mode == 2 || (mode == 1 && n_beta >= kDeviceDenseMinBetas));
   return RDM_OK;
 }
 
@@ -1829,7 +1851,8 @@ rdm_status EstimateRun::upload_betas() {
 
 rdm_status EstimateRun::fetch_dense() {
   std::vector<double> lohi(2 * (size_t)n_rec);
-  CK(cudaMemcpyAsync(cstore.data(), d_c, cstore.size() * sizeof(double), cudaMemcpyDeviceToHost, s));
+  if (!coef_on_device)
+    CK(cudaMemcpyAsync(cstore.data(), d_c, cstore.size() * sizeof(double), cudaMemcpyDeviceToHost, s));
   CK(cudaMemcpyAsync(lohi.data(), d_lohi, lohi.size() * sizeof(double), cudaMemcpyDeviceToHost, s));
   CK(cudaStreamSynchronize(s));
   d2h += (cstore.size() + lohi.size()) * sizeof(double);
@@ -1898,6 +1921,44 @@ static bool normalise_grams(const std::vector<double>& g, int n_beta, int n_v, i
   return ok;
 }
 
+// The Gram coefficients on the device: E in d_e, quad and the steps each beta needs back.
+rdm_status EstimateRun::device_coefficients(double e0, std::vector<double>& quad, std::vector<int>& kbeta) {
+  const size_t nq = (size_t)n_beta * n_v;
+  std::vector<double> f(nq);
+  for (int l = 0; l < n_v; ++l)
+    for (int bi = 0; bi < n_beta; ++bi) f[(size_t)l * n_beta + bi] = std::exp(-0.5 * betas[bi] * (tmin[l] - e0));
+  const double tau = gram_tau();
+  CoefJob j{};
+  j.k = k;
+  j.ng = ng;
+  j.n_v = n_v;
+  j.n_beta = n_beta;
+  j.tau2 = tau * tau;
+  j.c = d_c;
+  j.f = d_cheb;
+  j.mz = MZ(1);
+  j.e = d_e;
+  j.quad = d_cheb + nq;
+  j.kb = reinterpret_cast<int*>(j.quad + nq * nv);
+  j.jlast = j.kb + (n_beta + 1) / 2 * 2;
+  CK(cudaMemcpyAsync(d_cheb, f.data(), nq * sizeof(double), cudaMemcpyHostToDevice, s));
+  h2d += nq * sizeof(double);
+  CK(counted([&] { return launch_gram_coef(ds, j, s); }));
+  if (prof) prof->begin(kKSmall, s, false);  // (two launches)
+  std::vector<double> back(nq * nv + (size_t)(n_beta + 1) / 2);
+  CK(cudaMemcpyAsync(back.data(), j.quad, back.size() * sizeof(double), cudaMemcpyDeviceToHost, s));
+  CK(cudaStreamSynchronize(s));
+  d2h += back.size() * sizeof(double);
+  std::copy_n(back.data(), nq * nv, quad.data());
+  std::memcpy(kbeta.data(), back.data() + nq * nv, (size_t)n_beta * sizeof(int));
+  for (double x : quad)
+    if (!std::isfinite(x)) {
+      set_error("the device small dense step gave a non-finite coefficient");
+      return RDM_ENUMERIC;
+    }
+  return RDM_OK;
+}
+
 rdm_status EstimateRun::finish_rest() {
   rdm_status st = RDM_OK;
   const int n = k * ds;
@@ -1931,7 +1992,7 @@ rdm_status EstimateRun::finish_rest() {
   const size_t cstride_g = (size_t)ngo * nvo;
   const bool e_view = store;
   std::vector<double> quad((size_t)n_beta * n_v * nvo, 0.0), gram((size_t)n_beta * n_v * nvo, 0.0);
-  std::vector<double> hE(psz.e);
+  std::vector<double> hE(coef_on_device ? 0 : psz.e);
   std::vector<double> hg(psz.gram);
   // Trailing Krylov steps whose coefficient blocks are below the working precision
   // relative to the whole coefficient vector (|c_j| <= 1e-3 eps |c| for every vector, at
@@ -1939,16 +2000,16 @@ rdm_status EstimateRun::finish_rest() {
   // zero for that beta (so the result does not depend on how betas are chunked), and the
   // Gram pass (stored basis) or the recurrence of pass 2 stops after the last step any
   // beta of the chunk needs.
-  const double tau = 1e-3 * (o->precision == RDM_FP32 ? 1.1920928955078125e-07 : 2.220446049250313e-16);
+  const double tau = gram_tau();
   auto last_significant = [&](const std::vector<double>& c, int width) -> int {
     double tot = 0.0;
-    for (double x : c) tot += x * x;
+    for (double x : c) tot = std::fma(x, x, tot);
     int last = 0;
     for (int j = 0; j < k; ++j) {
       double sj = 0.0;
       for (int t = 0; t < ds * width; ++t) {
         const double x = c[(size_t)j * ds * width + t];
-        sj += x * x;
+        sj = std::fma(x, x, sj);
       }
       if (sj > tau * tau * tot) last = j + 1;
     }
@@ -1964,64 +2025,69 @@ rdm_status EstimateRun::finish_rest() {
   };
   for (int b0 = 0; b0 < n_beta; b0 += p.nbc) {
     const int nb = std::min(p.nbc, n_beta - b0);
-    std::fill(hE.begin(), hE.end(), 0.0);
-    std::fill(jlast.begin(), jlast.end(), 1);
-    const auto coef_t0 = std::chrono::steady_clock::now();
-    parallel_for(n_v, [&](int l) {
-      std::vector<double> c;
-      for (int bi = 0; bi < nb; ++bi) {
-        double* q = &quad[((size_t)(b0 + bi) * n_v + l) * nvo];
-        if (!p.single) {
-          coef_c(l, b0 + bi, c);
-          jlast[(size_t)bi * n_v + l] = last_significant(c, ds);
-          for (int a = 0; a < ds; ++a)
-            for (int b = 0; b < ds; ++b) {
-              double sacc = 0.0;
-              for (int r = 0; r < n; ++r) sacc += c[(size_t)r * ds + a] * c[(size_t)r * ds + b];
-              q[a * ds + b] = sacc;
-            }
-          for (int j = 0; j < k; ++j) {
-            const double* M = &mz[(size_t)j * cstride + (size_t)l * nv];
-            double* Ej = &hE[(((size_t)j * p.nbc + bi) * ng + l) * nv];
+    if (coef_on_device) {  // (the whole grid: a stored basis has one chunk)
+      st = device_coefficients(e0, quad, kbeta);
+      if (st != RDM_OK) return st;
+    } else {
+      std::fill(hE.begin(), hE.end(), 0.0);
+      std::fill(jlast.begin(), jlast.end(), 1);
+      const auto coef_t0 = std::chrono::steady_clock::now();
+      parallel_for(n_v, [&](int l) {
+        std::vector<double> c;
+        for (int bi = 0; bi < nb; ++bi) {
+          double* q = &quad[((size_t)(b0 + bi) * n_v + l) * nvo];
+          if (!p.single) {
+            coef_c(l, b0 + bi, c);
+            jlast[(size_t)bi * n_v + l] = last_significant(c, ds);
             for (int a = 0; a < ds; ++a)
               for (int b = 0; b < ds; ++b) {
                 double sacc = 0.0;
-                for (int m = 0; m < ds; ++m) sacc += M[a * ds + m] * c[(size_t)(j * ds + m) * ds + b];
-                Ej[a * ds + b] = sacc;
+                for (int r = 0; r < n; ++r) sacc = std::fma(c[(size_t)r * ds + a], c[(size_t)r * ds + b], sacc);
+                q[a * ds + b] = sacc;
               }
+            for (int j = 0; j < k; ++j) {
+              const double* M = &mz[(size_t)j * cstride + (size_t)l * nv];
+              double* Ej = &hE[(((size_t)j * p.nbc + bi) * ng + l) * nv];
+              for (int a = 0; a < ds; ++a)
+                for (int b = 0; b < ds; ++b) {
+                  double sacc = 0.0;
+                  for (int m = 0; m < ds; ++m) sacc = std::fma(M[a * ds + m], c[(size_t)(j * ds + m) * ds + b], sacc);
+                  Ej[a * ds + b] = sacc;
+                }
+            }
+            continue;
           }
-          continue;
+          for (int i = 0; i < dso; ++i) {  // single recurrences: column r = l dso + i
+            const int r = l * dso + i;
+            coef_c(r, b0 + bi, c);
+            int& jl = jlast[(size_t)bi * n_v + l];
+            jl = std::max(i == 0 ? 1 : jl, last_significant(c, 1));
+            double sacc = 0.0;
+            for (int m = 0; m < n; ++m) sacc += c[m] * c[m];
+            q[i * dso + i] = sacc;
+            for (int j = 0; j < k; ++j) {
+              const double e = mz[(size_t)j * cstride + r] * c[j];
+              if (e_view)
+                hE[(((size_t)j * p.nbc + bi) * ngo + l) * nvo + i * dso + i] = e;
+              else
+                hE[((size_t)j * p.nbc + bi) * ng + r] = e;
+            }
+          }
         }
-        for (int i = 0; i < dso; ++i) {  // single recurrences: column r = l dso + i
-          const int r = l * dso + i;
-          coef_c(r, b0 + bi, c);
-          int& jl = jlast[(size_t)bi * n_v + l];
-          jl = std::max(i == 0 ? 1 : jl, last_significant(c, 1));
-          double sacc = 0.0;
-          for (int m = 0; m < n; ++m) sacc += c[m] * c[m];
-          q[i * dso + i] = sacc;
-          for (int j = 0; j < k; ++j) {
-            const double e = mz[(size_t)j * cstride + r] * c[j];
-            if (e_view)
-              hE[(((size_t)j * p.nbc + bi) * ngo + l) * nvo + i * dso + i] = e;
-            else
-              hE[((size_t)j * p.nbc + bi) * ng + r] = e;
-          }
+      });
+      host_ms += std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - coef_t0).count();
+      for (int bi = 0; bi < nb; ++bi) {
+        const int kb =
+            std::max(1, *std::max_element(jlast.begin() + (size_t)bi * n_v, jlast.begin() + (size_t)(bi + 1) * n_v));
+        kbeta[bi] = kb;
+        for (int j = kb; j < k; ++j) {  // E_j of this beta beyond its last needed step
+          double* e0p = &hE[((size_t)j * p.nbc + bi) * (e_view ? ngo * nvo : ng * nv)];
+          std::fill(e0p, e0p + (size_t)(e_view ? ngo * nvo : ng * nv), 0.0);
         }
       }
-    });
-    host_ms += std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - coef_t0).count();
-    for (int bi = 0; bi < nb; ++bi) {
-      const int kb =
-          std::max(1, *std::max_element(jlast.begin() + (size_t)bi * n_v, jlast.begin() + (size_t)(bi + 1) * n_v));
-      kbeta[bi] = kb;
-      for (int j = kb; j < k; ++j) {  // E_j of this beta beyond its last needed step
-        double* e0p = &hE[((size_t)j * p.nbc + bi) * (e_view ? ngo * nvo : ng * nv)];
-        std::fill(e0p, e0p + (size_t)(e_view ? ngo * nvo : ng * nv), 0.0);
-      }
+      CK(cudaMemcpyAsync(d_e, hE.data(), hE.size() * sizeof(double), cudaMemcpyHostToDevice, s));
+      h2d += hE.size() * sizeof(double);
     }
-    CK(cudaMemcpyAsync(d_e, hE.data(), hE.size() * sizeof(double), cudaMemcpyHostToDevice, s));
-    h2d += hE.size() * sizeof(double);
     if (store) {
       // ---- psi = sum_j W_j E_j over the stored blocks, Gram fused (Gram view).
       const int gmax = gram_betas(pstride_g, nb);

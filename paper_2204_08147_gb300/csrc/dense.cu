@@ -36,6 +36,7 @@
 
 #include <algorithm>
 #include <mutex>
+#include <type_traits>
 #include <vector>
 
 #include "rdm_internal.h"
@@ -347,6 +348,79 @@ __global__ void __launch_bounds__(kChebThreads) k_cheb_combine(const DenseJob* j
   }
 }
 
+// The Gram coefficients of bath vector blockIdx.x at beta blockIdx.y from the combination
+// kernel's results, as the host forms them (the same products and sums in the same order):
+// c = f c0 with f = exp(-beta (t - E0) / 2), quad = c^T c, E_j = M_j c_j, and the last step j
+// with |c_j|^2 > tau2 |c|^2. Blocks past the real vectors write zero E (padding). The two long
+// sums run in one thread each (their order), the rest over the block.
+constexpr int kCoefThreads = 128;
+template <int DS>
+__global__ void __launch_bounds__(kCoefThreads) k_gram_coef(CoefJob J) {
+  constexpr int NV = DS * DS;
+  extern __shared__ __align__(16) double sc[];  // c [k * NV], |c_j|^2 [k]
+  __shared__ double tot;
+  __shared__ int last;
+  const int l = blockIdx.x, bi = blockIdx.y, k = J.k, ne = k * NV;
+  double* const sj = sc + ne;
+  const bool real = l < J.n_v;
+  if (real) {
+    const double f = J.f[(size_t)l * J.n_beta + bi];
+    const double* src = J.c + ((size_t)l * J.n_beta + bi) * ne;
+    for (int i = threadIdx.x; i < ne; i += kCoefThreads) sc[i] = __dmul_rn(f, src[i]);
+    if (threadIdx.x == 0) last = 0;
+    __syncthreads();
+  }
+  for (int i = threadIdx.x; i < ne; i += kCoefThreads) {
+    const int j = i / NV, a = i % NV / DS, b = i % DS;
+    double s = 0.0;
+    if (real) {
+      const double* M = J.mz + ((size_t)j * J.ng + l) * NV;
+#pragma unroll
+      for (int m = 0; m < DS; ++m) s = fma(M[a * DS + m], sc[(j * DS + m) * DS + b], s);
+    }
+    J.e[(((size_t)j * J.n_beta + bi) * J.ng + l) * NV + a * DS + b] = s;
+  }
+  if (!real) return;
+  if ((int)threadIdx.x < NV) {
+    const int a = threadIdx.x / DS, b = threadIdx.x % DS;
+    double s = 0.0;
+    for (int r = 0; r < k * DS; ++r) s = fma(sc[r * DS + a], sc[r * DS + b], s);
+    J.quad[((size_t)bi * J.n_v + l) * NV + threadIdx.x] = s;
+  } else if (threadIdx.x == 32) {
+    double s = 0.0;
+    for (int i = 0; i < ne; ++i) s = fma(sc[i], sc[i], s);
+    tot = s;
+  } else if (threadIdx.x >= 64) {
+    for (int j = threadIdx.x - 64; j < k; j += kCoefThreads - 64) {
+      double s = 0.0;
+      for (int t = 0; t < NV; ++t) s = fma(sc[j * NV + t], sc[j * NV + t], s);
+      sj[j] = s;
+    }
+  }
+  __syncthreads();
+  for (int j = threadIdx.x; j < k; j += kCoefThreads)
+    if (sj[j] > __dmul_rn(J.tau2, tot)) atomicMax(&last, j + 1);
+  __syncthreads();
+  if (threadIdx.x == 0) J.jlast[(size_t)bi * J.n_v + l] = last;
+}
+
+// kb[beta] = the last step any vector needs (at least 1); E beyond it is zeroed.
+template <int DS>
+__global__ void __launch_bounds__(256) k_gram_coef_tail(CoefJob J) {
+  __shared__ int kb;
+  const int bi = blockIdx.x;
+  if (threadIdx.x == 0) kb = 1;
+  __syncthreads();
+  int m = 1;
+  for (int l = threadIdx.x; l < J.n_v; l += 256) m = max(m, J.jlast[(size_t)bi * J.n_v + l]);
+  atomicMax(&kb, m);
+  __syncthreads();
+  if (threadIdx.x == 0) J.kb[bi] = kb;
+  const int per = J.ng * DS * DS;
+  for (int j = kb; j < J.k; ++j)
+    for (int i = threadIdx.x; i < per; i += 256) J.e[((size_t)j * J.n_beta + bi) * per + i] = 0.0;
+}
+
 template <int DS>
 cudaError_t launch_dense(const DenseJob* jobs, const int* pre, int n_jobs, int n_blocks, int max_k,
                          int max_beta_chunks, int max_vstride, cudaStream_t st) {
@@ -375,6 +449,23 @@ cudaError_t launch_dense(const DenseJob* jobs, const int* pre, int n_jobs, int n
 }
 
 }  // namespace
+
+cudaError_t launch_gram_coef(int ds, const CoefJob& j, cudaStream_t st) {
+  if (j.k < 1 || j.n_beta < 1 || j.n_beta > 65535 || j.n_v < 1 || j.n_v > j.ng || !dense_device_fits(j.k, ds))
+    return cudaErrorInvalidValue;
+  const size_t sm = ((size_t)j.k * ds * ds + j.k) * sizeof(double);  // at most 45 KB (dense_device_fits)
+  const dim3 grid((unsigned)j.ng, (unsigned)j.n_beta);
+  auto go = [&](auto d) {
+    constexpr int DS = decltype(d)::value;
+    k_gram_coef<DS><<<grid, kCoefThreads, sm, st>>>(j);
+    k_gram_coef_tail<DS><<<j.n_beta, 256, 0, st>>>(j);
+    return cudaGetLastError();
+  };
+  if (ds == 1) return go(std::integral_constant<int, 1>{});
+  if (ds == 2) return go(std::integral_constant<int, 2>{});
+  if (ds == 4) return go(std::integral_constant<int, 4>{});
+  return cudaErrorInvalidValue;
+}
 
 bool dense_device_fits(int k, int ds) {
   const size_t smv = (size_t)5 * k * ds * ds * sizeof(double);

@@ -350,6 +350,23 @@ size_t dense_jobs_bytes(int n_jobs);
 // One launch of each dense kernel over all recurrences of all jobs (same d_s).
 cudaError_t launch_dense_jobs(int ds, const DenseJob* host_jobs, int n_jobs, void* scratch, cudaStream_t st);
 
+// The Gram coefficients of one estimate (block recurrences, every beta) on the device, from
+// the device small dense step's c: see k_gram_coef. c: [vector][beta][k d_s][d_s]; f:
+// [vector][beta]; mz: M_1..M_k [step][ng][d_s^2]; out e [step][beta][ng][d_s^2], quad
+// [beta][vector][d_s^2], jlast [beta][vector] (scratch), kb [beta].
+struct CoefJob {
+  int k, ng, n_v, n_beta;
+  double tau2;
+  const double* c;
+  const double* f;
+  const double* mz;
+  double* e;
+  double* quad;
+  int* jlast;
+  int* kb;
+};
+cudaError_t launch_gram_coef(int ds, const CoefJob& j, cudaStream_t st);
+
 constexpr uint32_t kFlagNonFinite = 0x100u;
 
 }  // namespace rdm

@@ -39,3 +39,24 @@ def test_gram_beta_groups(lib, n, n_sys, n_v, n_beta):
         np.testing.assert_allclose(grid["rho"], grid["rho_quad"], atol=1e-4, rtol=0)
     finally:
         ctx.close()
+
+
+@pytest.mark.parametrize("n,n_sys,n_v,k", [(8, 1, 3, 1), (9, 0, 5, 7), (10, 2, 3, 40), (11, 1, 9, 33), (12, 2, 64, 12)])
+@pytest.mark.parametrize("prec", ["fp32", "fp64"])
+def test_coefficients_on_the_device_are_the_hosts(lib, n, n_sys, n_v, k, prec):
+    """With the basis stored, the Gram coefficients of a grid of 8 or more betas are formed
+    on the device from the device small dense step; with the basis recomputed, on the host
+    from the same step. The same products and sums in the same order: the same bits in the
+    Gram and quadrature forms of every vector."""
+    spec = W.random_model(n, n_sys, 17)
+    ctx = lib.Context(0)
+    try:
+        ham = lib.Hamiltonian(ctx, spec)
+        out = [ham.estimate(W.beta_grid(9, 0.02, 8.0), n_v, k, 4, precision=prec, dist="rademacher", full=True,
+                            passes=p) for p in ("store", "recompute")]
+        for key in ("quad_l", "gram_l", "rho", "lnZ", "rho_quad", "t_a", "t_b"):
+            np.testing.assert_array_equal(out[0][key], out[1][key])
+        slim = ham.estimate(W.beta_grid(9, 0.02, 8.0), n_v, k, 4, precision=prec, dist="rademacher")
+        np.testing.assert_array_equal(slim["rho"], out[0]["rho"])
+    finally:
+        ctx.close()
