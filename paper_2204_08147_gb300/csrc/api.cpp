@@ -4,6 +4,7 @@
 #include <sched.h>
 
 #include <algorithm>
+#include <array>
 #include <chrono>
 #include <atomic>
 #include <cmath>
@@ -1459,6 +1460,13 @@ class EstimateRun {
   PackedItem packed_item() const;
   const Plan& plan() const { return p; }
   bool packed_done = false;  // the first pass ran in a packed launch
+  // Before prepare(): the first pass may run in clusters (k_pass1_cluster); after it,
+  // whether it does.
+  bool in_clusters = false;
+  // float32 blocks of the tiled SpMM: their own launches are faster than the packed
+  // launch's untiled units (N = 15, 16 of the serving mix: a burst of 24 requests, N 12-16,
+  // 206 -> 131 ms).
+  bool tiled_launches() const { return sa.tile_k != nullptr && !in_clusters && L.precision == RDM_FP32; }
 
  private:
   rdm_ham* ham;
@@ -1543,6 +1551,32 @@ class EstimateRun {
 };
 
 constexpr size_t kPackedMaxBlock = size_t(64) << 20;
+
+// A stream beside another: fork makes it wait for what `s` holds, join makes `s` wait for it.
+struct SideStream {
+  cudaStream_t stream = nullptr;
+  cudaEvent_t ev = nullptr;
+  bool open = false;
+  cudaError_t fork(cudaStream_t s) {
+    cudaError_t e = cudaStreamCreateWithFlags(&stream, cudaStreamNonBlocking);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaEventRecord(ev, s);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(stream, ev, 0);
+    open = e == cudaSuccess;
+    return e;
+  }
+  cudaError_t join(cudaStream_t s) {
+    cudaError_t e = cudaEventRecord(ev, stream);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(s, ev, 0);
+    if (e == cudaSuccess) open = false;
+    return e;
+  }
+  ~SideStream() {
+    if (stream && open) cudaStreamSynchronize(stream);  // fork without join: a failed launch
+    if (ev) cudaEventDestroy(ev);
+    if (stream) cudaStreamDestroy(stream);  // (its work completes first)
+  }
+};
 // Estimates whose blocks have fewer 1024-state tiles (all slices together) run the plain
 // SpMM (rdm_set_spmm_form).
 constexpr int64_t kTiledMinTiles = 32;
@@ -1648,7 +1682,8 @@ rdm_status EstimateRun::prepare(char* ws, size_t ws_bytes) {
     // 8 tiles (c1: 12 vs 31 us per launch), tiled faster from 64 tiles on.
     const int64_t tiles = p.tk_bytes ? ((int64_t)L.n_slices << (L.n_bits - kTileBits)) : 0;
     const int form = ham->ctx ? ham->ctx->spmm_form : 0;  // (the serving loop's own Hamiltonians have none)
-    sa.tile_k = p.tk_bytes && (form == 1 || (form == 0 && tiles >= kTiledMinTiles)) ? d_tk : nullptr;
+    in_clusters = in_clusters && packable() && pass1_cluster_fits(L, ham->tiled);
+    sa.tile_k = p.tk_bytes && (in_clusters || form == 1 || (form == 0 && tiles >= kTiledMinTiles)) ? d_tk : nullptr;
   }
   sa.err = d_flags + 1;
 
@@ -2520,6 +2555,90 @@ static rdm_status run_packed(rdm_ctx* ctx, cudaStream_t s, std::vector<EstimateR
   return RDM_OK;
 }
 
+// The first passes of `runs` in clusters: one launch per (d_s, tiles per slice), the
+// launches side by side on a few streams (on s alone while launches are timed), joined
+// before return. meta: device scratch for the descriptors (packed_meta_bytes of each group);
+// *used: bytes of it taken. keep: the descriptors' host images, which must outlive the work.
+static rdm_status run_clusters(cudaStream_t s, const std::vector<EstimateRun*>& runs, char* meta, size_t* used,
+                               std::vector<std::vector<char>>* keep, Profiler* prof) {
+  struct Group {
+    int ds, c_log, n_slices = 0, k = 0;
+    size_t smem = 0;
+    double bytes = 0.0;
+    std::vector<PackedItem> items;
+    std::vector<int> pre{0};
+  };
+  std::map<std::pair<int, int>, Group> groups;
+  for (const EstimateRun* r : runs) {
+    const PackedItem it = r->packed_item();
+    const std::pair<int, int> key(it.L.DS, it.L.n_bits - kTileBits);
+    Group& g = groups[key];
+    g.ds = key.first;
+    g.c_log = key.second;
+    g.items.push_back(it);
+    g.n_slices += it.L.n_slices;
+    g.pre.push_back(g.n_slices);
+    g.k = std::max(g.k, it.k);
+    g.smem = std::max(g.smem, pass1_cluster_smem(it.sa.tiled));
+    g.bytes += 6.0 * (double)it.L.block_bytes() * it.k;
+  }
+  // the longest launches first (steps times blocks)
+  std::vector<Group*> order;
+  for (auto& kv : groups) order.push_back(&kv.second);
+  std::stable_sort(order.begin(), order.end(), [](const Group* x, const Group* y) {
+    return ((int64_t)x->k * x->n_slices << x->c_log) > ((int64_t)y->k * y->n_slices << y->c_log);
+  });
+  const bool timing = prof && prof->on;
+  std::array<SideStream, 3> side;
+  int n_side = 0;
+  rdm_status st = RDM_OK;
+  for (size_t q = 0; q < order.size() && st == RDM_OK; ++q) {
+    Group& g = *order[q];
+    // (launches of items with different k do not need the k-sorted order of the packed grid)
+    const size_t o_pre = sizeof(PackedItem) * g.items.size();
+    std::vector<char> img(o_pre + sizeof(int) * g.pre.size());
+    std::memcpy(img.data(), g.items.data(), o_pre);
+    std::memcpy(img.data() + o_pre, g.pre.data(), sizeof(int) * g.pre.size());
+    char* dev = meta + *used;
+    *used += packed_meta_bytes((int)g.items.size(), g.k);
+    cudaStream_t ls = s;
+    if (!timing && q > 0) {
+      const int w = (int)((q - 1) % side.size());
+      if (w >= n_side) {
+        if (side[w].fork(s) != cudaSuccess) {
+          set_error("batch: no side stream: %s", cudaGetErrorString(cudaGetLastError()));
+          st = RDM_ECUDA;
+          break;
+        }
+        n_side = w + 1;
+      }
+      ls = side[w].stream;
+    }
+    PackedPlan pp{};
+    pp.items = reinterpret_cast<const PackedItem*>(dev);
+    pp.n_items = (int)g.items.size();
+    pp.k_max = g.k;
+    pp.pre_slices = reinterpret_cast<const int*>(dev + o_pre);
+    cudaError_t e = cudaMemcpyAsync(dev, img.data(), img.size(), cudaMemcpyHostToDevice, ls);
+    keep->push_back(std::move(img));
+    const int ev = prof ? prof->begin(kKPacked, ls, true) : -1;
+    if (e == cudaSuccess) e = launch_pass1_cluster(g.ds, pp, g.c_log, g.n_slices, g.smem, ls);
+    if (prof) prof->end(kKPacked, ev, ls, g.bytes);
+    if (e != cudaSuccess) {
+      set_error("first pass in clusters: %s", cudaGetErrorString(e));
+      st = RDM_ECUDA;
+    }
+  }
+  for (int w = 0; w < n_side; ++w) {
+    const cudaError_t e = side[w].join(s);
+    if (e != cudaSuccess && st == RDM_OK) {
+      set_error("batch: %s", cudaGetErrorString(e));
+      st = RDM_ECUDA;
+    }
+  }
+  return st;
+}
+
 rdm_status estimate_batch_impl(rdm_ctx* ctx, cudaStream_t s, char* ws, size_t ws_bytes,
                                rdm_batch_item* items, int n, const size_t* need, Profiler* prof) {
   std::vector<std::unique_ptr<EstimateRun>> runs(n);
@@ -2531,28 +2650,57 @@ rdm_status estimate_batch_impl(rdm_ctx* ctx, cudaStream_t s, char* ws, size_t ws
   char* meta = ws;
   off = 6 * meta_b + dense_jobs_bytes(n);
   rdm_status first_bad = RDM_OK;
+  bool clusters = true;  // (a packed_form other than 0 asks for the untiled units)
+  if (ctx) {
+    std::lock_guard<std::mutex> lk(ctx->tuning.mu);
+    clusters = ctx->packed_form == 0;
+  }
   for (int i = 0; i < n; ++i) {
     rdm_batch_item& it = items[i];
     runs[i] = std::make_unique<EstimateRun>(it.ham, s, it.betas, it.n_beta, it.n_v, it.k, it.seed, &it.opts,
                                             it.out, prof);
+    runs[i]->in_clusters = clusters;
     it.status = runs[i]->prepare(ws + off, need[i]);
     off += need[i];
     if (it.status != RDM_OK && first_bad == RDM_OK) first_bad = it.status;
   }
-  // packed first passes, one launch per (precision, d_s)
-  int slot = 0;
+  // First passes in clusters, and the others packed, one launch per (precision, d_s). The
+  // descriptors of all groups take less than the 6 meta_b: the groups part the items.
+  size_t meta_off = 0;
+  std::vector<std::vector<char>> keep;
+  {
+    std::vector<EstimateRun*> group;
+    std::vector<int> idx;
+    for (int i = 0; i < n; ++i)
+      if (items[i].status == RDM_OK && runs[i]->in_clusters) {
+        group.push_back(runs[i].get());
+        idx.push_back(i);
+      }
+    if (!group.empty()) {
+      const rdm_status st = run_clusters(s, group, meta, &meta_off, &keep, prof);
+      for (int i : idx) {
+        if (st != RDM_OK) items[i].status = st;
+        runs[i]->packed_done = true;
+      }
+      if (st != RDM_OK && first_bad == RDM_OK) first_bad = st;
+    }
+  }
   for (int prec : {RDM_FP32, RDM_FP64})
     for (int ds : {1, 2, 4}) {
       std::vector<EstimateRun*> group;
       std::vector<int> idx;
       for (int i = 0; i < n; ++i)
-        if (items[i].status == RDM_OK && runs[i]->packable() && runs[i]->plan().L.precision == prec &&
-            runs[i]->plan().L.DS == ds) {
+        if (items[i].status == RDM_OK && runs[i]->packable() && !runs[i]->in_clusters &&
+            !(clusters && runs[i]->tiled_launches()) &&
+            runs[i]->plan().L.precision == prec && runs[i]->plan().L.DS == ds) {
           group.push_back(runs[i].get());
           idx.push_back(i);
         }
       if (group.empty()) continue;
-      const rdm_status st = run_packed(ctx, s, group, prec, ds, meta + (size_t)slot++ * meta_b, prof);
+      int group_k = 1;
+      for (int i : idx) group_k = std::max(group_k, items[i].k);
+      const rdm_status st = run_packed(ctx, s, group, prec, ds, meta + meta_off, prof);
+      meta_off += packed_meta_bytes((int)group.size(), group_k);
       if (st != RDM_OK)
         for (int i : idx) {
           items[i].status = st;

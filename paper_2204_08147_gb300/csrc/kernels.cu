@@ -669,6 +669,109 @@ __device__ __forceinline__ void reg_lanes(T (&y)[RPT][VW], const T (&x)[RPT][VW]
   if (__any_sync(0xffffffffu, in_use(c_odd))) reg_half<K, 1>(y, x, c_odd);
 }
 
+// The in-tile terms: y += (terms) x, xo the thread's own rows of the tile `own`.
+template <bool UNI, int RG, int STEP, typename T, int VW, int RPT>
+__device__ __forceinline__ void own_terms(T (&y)[RPT][VW], const T (&xo)[RPT][VW], const T* own, int rgoff,
+                                          const TiledTerms& tt, const T* s_reg, const GrpS<T>* grp,
+                                          const LaneS<T>* lanet, uint32_t act_lane, uint32_t act_grp) {
+  const uint32_t reg_flags = tt.reg_flags;
+  // fields and hops of the register rows alone
+  if (reg_flags & 2u) reg_uniform<1>(y, xo, s_reg[8 + 1], s_reg[1]);
+  if (reg_flags & 4u) reg_uniform<2>(y, xo, s_reg[8 + 2], s_reg[2]);
+  if (reg_flags & 16u) reg_uniform<4>(y, xo, s_reg[8 + 4], s_reg[4]);
+  if constexpr (!UNI) {
+    if (reg_flags & 8u) reg_uniform<3>(y, xo, s_reg[8 + 3], s_reg[3]);
+    if (reg_flags & 32u) reg_uniform<5>(y, xo, s_reg[8 + 5], s_reg[5]);
+    if (reg_flags & 64u) reg_uniform<6>(y, xo, s_reg[8 + 6], s_reg[6]);
+  } else if (reg_flags & (8u | 32u | 64u)) {
+    reg_uniform<3>(y, xo, s_reg[8 + 3], s_reg[3]);
+    reg_uniform<5>(y, xo, s_reg[8 + 5], s_reg[5]);
+    reg_uniform<6>(y, xo, s_reg[8 + 6], s_reg[6]);
+  }
+  // a row-group spin's field and its hops with the register spins share one set of loads
+  for (int t = 0; t < tt.n_grp; ++t) {
+    const GrpS<T>& G = grp[t];
+    const bool odd = (act_grp >> t) & 1u;
+    const uint32_t fl = G.flags;
+    T xp[RPT][VW];
+    load_rows<STEP>(xp, own + (rgoff ^ (int)G.off));
+    if (fl & kPatField) {
+      const T c = G.cf;
+#pragma unroll
+      for (int m = 0; m < RPT; ++m) axpy(y[m], c, xp[m]);
+    }
+    if (fl & kPatReg) reg_lanes<1>(y, xp, odd ? G.co[0] : G.ce[0], odd ? G.ce[0] : G.co[0]);
+    if (fl & (kPatReg << 1)) reg_lanes<2>(y, xp, odd ? G.co[1] : G.ce[1], odd ? G.ce[1] : G.co[1]);
+    if (fl & (kPatReg << 2)) reg_lanes<4>(y, xp, odd ? G.co[2] : G.ce[2], odd ? G.ce[2] : G.co[2]);
+  }
+  // terms of the row-group spins alone
+  if constexpr (UNI) {
+    int t = 0;
+    for (; t + 1 < tt.n_own; t += 2)
+      rows_fma2<STEP>(y, own + (rgoff ^ (int)lanet[t].off), lanet[t].co, own + (rgoff ^ (int)lanet[t + 1].off),
+                       lanet[t + 1].co);
+    if (t < tt.n_own) rows_fma<STEP>(y, own + (rgoff ^ (int)lanet[t].off), lanet[t].co);
+  } else {
+    for (int t = 0; t < tt.n_own; ++t) {
+      const LaneS<T> d = lanet[t];
+      const T c = ((act_lane >> t) & 1u) ? d.co : d.ce;
+      // where the coefficient differs across the warp's lanes they all run the term
+      if (__any_sync(0xffffffffu, in_use(c))) rows_fma<STEP>(y, own + (rgoff ^ (int)d.off), c);
+    }
+  }
+}
+// The terms of one high spin on its partner tile P: its field and its hops with in-tile
+// spins (hs: whether it is down here).
+template <bool UNI, int STEP, typename T, int VW, int RPT>
+__device__ __forceinline__ void single_terms(T (&y)[RPT][VW], const T* P, int rgoff, int rg, const PatS<T>& A, bool hs,
+                                             const LaneS<T>* lanet) {
+  const uint32_t fl = A.flags;
+  if (fl & (kPatField | (kPatReg * 7u))) {
+    T xp[RPT][VW];
+    load_rows<STEP>(xp, P + rgoff);
+    if (fl & kPatField) {
+      const T c = A.cf;
+#pragma unroll
+      for (int m = 0; m < RPT; ++m) axpy(y[m], c, xp[m]);
+    }
+    if (fl & kPatReg) reg_uniform<1>(y, xp, hs ? A.co[0] : A.ce[0], hs ? A.ce[0] : A.co[0]);
+    if (fl & (kPatReg << 1)) reg_uniform<2>(y, xp, hs ? A.co[1] : A.ce[1], hs ? A.ce[1] : A.co[1]);
+    if (fl & (kPatReg << 2)) reg_uniform<4>(y, xp, hs ? A.co[2] : A.ce[2], hs ? A.ce[2] : A.co[2]);
+  }
+  for (int t = A.start; t < A.end; ++t) {
+    const LaneS<T> d = lanet[t];
+    const bool odd = (((uint32_t)rg & d.low) != 0u) != hs;
+    const T c = UNI || odd ? d.co : d.ce;
+    if (UNI || __any_sync(0xffffffffu, in_use(c))) rows_fma<STEP>(y, P + (rgoff ^ (int)d.off), c);
+  }
+}
+// An opposite-spin pair: term l of group A (its spin down here, tile Z) acts on the rows
+// whose spin l is up, of group B (spin up, tile O) on the others, so every row takes exactly
+// one of the two.
+template <int STEP, typename T, int VW, int RPT>
+__device__ __forceinline__ void pair_terms(T (&y)[RPT][VW], const T* Z, const T* O, int rgoff, int rg,
+                                           const PatS<T>& A, const PatS<T>& B, const LaneS<T>* lanet) {
+  const uint32_t fl = A.flags;
+  if (fl & (kPatReg * 7u)) {
+    T xp[RPT][VW];
+    load_rows<STEP>(xp, Z + rgoff);
+    if (fl & kPatReg) reg_half<1, 1>(y, xp, A.co[0]);
+    if (fl & (kPatReg << 1)) reg_half<2, 1>(y, xp, A.co[1]);
+    if (fl & (kPatReg << 2)) reg_half<4, 1>(y, xp, A.co[2]);
+    load_rows<STEP>(xp, O + rgoff);
+    if (fl & kPatReg) reg_half<1, 0>(y, xp, B.co[0]);
+    if (fl & (kPatReg << 1)) reg_half<2, 0>(y, xp, B.co[1]);
+    if (fl & (kPatReg << 2)) reg_half<4, 0>(y, xp, B.co[2]);
+  }
+  const int n = A.end - A.start;
+  const LaneS<T>* const la = lanet + A.start;
+  const LaneS<T>* const lb = lanet + B.start;
+  for (int t = 0; t < n; ++t) {
+    const bool up = ((uint32_t)rg & la[t].low) != 0u;
+    rows_fma<STEP>(y, (up ? Z : O) + (rgoff ^ (int)la[t].off), up ? la[t].co : lb[t].co);
+  }
+}
+
 // Diagonal of H on this thread's RPT rows rg + RG m of a tile, from the tile's A-table
 // row hk (TileDiag): low[r] + sum_q A_q (-1)^popc(q & m), one RPT-point Walsh-Hadamard
 // transform of the A_q.
@@ -690,6 +793,49 @@ __device__ __forceinline__ void tile_diagonal(T (&dg)[RPT], const T* low, const 
       }
 #pragma unroll
   for (int m = 0; m < RPT; ++m) dg[m] = low[rg + RG * m] + A[m];
+}
+
+// The term tables into shared memory, by all threads of the block.
+template <int BS, typename T>
+__device__ __forceinline__ void load_tables(const TiledTerms& tt, PatS<T>* pat, GrpS<T>* grp, LaneS<T>* lanet, T* s_reg,
+                                            T* s_low) {
+  for (int i = threadIdx.x; i < tt.n_part; i += blockDim.x) {
+    PatS<T> r;
+    const double* c = tt.pat_coef + (size_t)i * 7;
+    r.high = tt.pat_high[i];
+    r.flags = tt.pat_flags[i];
+    r.start = tt.pat_start[i];
+    r.end = tt.pat_start[i + 1];
+    r.cf = (T)c[0];
+    for (int q = 0; q < 3; ++q) {
+      r.co[q] = (T)c[1 + q];
+      r.ce[q] = (T)c[4 + q];
+    }
+    pat[i] = r;
+  }
+  for (int i = threadIdx.x; i < tt.n_grp; i += blockDim.x) {
+    GrpS<T> r;
+    const double* c = tt.grp_coef + (size_t)i * 7;
+    r.low = tt.grp_low[i];
+    r.off = r.low * BS;
+    r.flags = tt.grp_flags[i];
+    r.cf = (T)c[0];
+    for (int q = 0; q < 3; ++q) {
+      r.co[q] = (T)c[1 + q];
+      r.ce[q] = (T)c[4 + q];
+    }
+    grp[i] = r;
+  }
+  for (int i = threadIdx.x; i < tt.n_lane; i += blockDim.x) {
+    LaneS<T> r;
+    r.co = (T)tt.lane_coef[2 * i];
+    r.ce = (T)tt.lane_coef[2 * i + 1];
+    r.low = tt.lane_low[i];
+    r.off = r.low * BS;
+    lanet[i] = r;
+  }
+  for (int i = threadIdx.x; i < 16; i += blockDim.x) s_reg[i] = (T)tt.reg_coef[i];
+  for (int i = threadIdx.x; i < kTileRows; i += blockDim.x) s_low[i] = (T)tt.dg.low[i];
 }
 
 template <typename T, int DS, int MODE, bool UNI = false>
@@ -733,43 +879,7 @@ __global__ void __launch_bounds__(kTiledThreads, 1) k_spmm_tiled(Layout L, SpmmA
   T* const s_reg = reinterpret_cast<T*>(lanet + nlane);  // [8] c_odd, [8] c_even
   T* const s_low = s_reg + 16;
 
-  for (int i = threadIdx.x; i < npart; i += blockDim.x) {
-    PatS<T> r;
-    const double* c = tt.pat_coef + (size_t)i * 7;
-    r.high = tt.pat_high[i];
-    r.flags = tt.pat_flags[i];
-    r.start = tt.pat_start[i];
-    r.end = tt.pat_start[i + 1];
-    r.cf = (T)c[0];
-    for (int q = 0; q < 3; ++q) {
-      r.co[q] = (T)c[1 + q];
-      r.ce[q] = (T)c[4 + q];
-    }
-    pat[i] = r;
-  }
-  for (int i = threadIdx.x; i < tt.n_grp; i += blockDim.x) {
-    GrpS<T> r;
-    const double* c = tt.grp_coef + (size_t)i * 7;
-    r.low = tt.grp_low[i];
-    r.off = r.low * BS;
-    r.flags = tt.grp_flags[i];
-    r.cf = (T)c[0];
-    for (int q = 0; q < 3; ++q) {
-      r.co[q] = (T)c[1 + q];
-      r.ce[q] = (T)c[4 + q];
-    }
-    grp[i] = r;
-  }
-  for (int i = threadIdx.x; i < nlane; i += blockDim.x) {
-    LaneS<T> r;
-    r.co = (T)tt.lane_coef[2 * i];
-    r.ce = (T)tt.lane_coef[2 * i + 1];
-    r.low = tt.lane_low[i];
-    r.off = r.low * BS;
-    lanet[i] = r;
-  }
-  for (int i = threadIdx.x; i < 16; i += blockDim.x) s_reg[i] = (T)tt.reg_coef[i];
-  for (int i = threadIdx.x; i < kTileRows; i += blockDim.x) s_low[i] = (T)tt.dg.low[i];
+  load_tables<BS>(tt, pat, grp, lanet, s_reg, s_low);
   if (threadIdx.x == 0) {
     for (int i = 0; i < kStages; ++i) {
       mbar_init(&full[i], 1);
@@ -962,7 +1072,6 @@ __global__ void __launch_bounds__(kTiledThreads, 1) k_spmm_tiled(Layout L, SpmmA
   uint32_t act_lane = 0u, act_grp = 0u;
   for (int t = 0; t < tt.n_own; ++t) act_lane |= (uint32_t)(__popc((uint32_t)rg & lanet[t].low) & 1) << t;
   for (int t = 0; t < tt.n_grp; ++t) act_grp |= (uint32_t)(((uint32_t)rg & grp[t].low) != 0u) << t;
-  const uint32_t reg_flags = tt.reg_flags;
 
   // The consumers walk the same (slice, tile) sequence as the producers. At every
   // change of slice (and at the end) they close the finished slice; every consumer
@@ -1048,73 +1157,12 @@ __global__ void __launch_bounds__(kTiledThreads, 1) k_spmm_tiled(Layout L, SpmmA
 #pragma unroll
         for (int v = 0; v < VW; ++v) y[m][v] = dg[m] * xo[m][v];
     }
-    // fields and hops of the register rows alone
-    if (reg_flags & 2u) reg_uniform<1>(y, xo, s_reg[8 + 1], s_reg[1]);
-    if (reg_flags & 4u) reg_uniform<2>(y, xo, s_reg[8 + 2], s_reg[2]);
-    if (reg_flags & 16u) reg_uniform<4>(y, xo, s_reg[8 + 4], s_reg[4]);
-    if constexpr (!UNI) {
-      if (reg_flags & 8u) reg_uniform<3>(y, xo, s_reg[8 + 3], s_reg[3]);
-      if (reg_flags & 32u) reg_uniform<5>(y, xo, s_reg[8 + 5], s_reg[5]);
-      if (reg_flags & 64u) reg_uniform<6>(y, xo, s_reg[8 + 6], s_reg[6]);
-    } else if (reg_flags & (8u | 32u | 64u)) {
-      reg_uniform<3>(y, xo, s_reg[8 + 3], s_reg[3]);
-      reg_uniform<5>(y, xo, s_reg[8 + 5], s_reg[5]);
-      reg_uniform<6>(y, xo, s_reg[8 + 6], s_reg[6]);
-    }
-    // a row-group spin's field and its hops with the register spins share one set of loads
-    for (int t = 0; t < tt.n_grp; ++t) {
-      const GrpS<T>& G = grp[t];
-      const bool odd = (act_grp >> t) & 1u;
-      const uint32_t fl = G.flags;
-      T xp[RPT][VW];
-      load_rows<kStep>(xp, own + (rgoff ^ (int)G.off));
-      if (fl & kPatField) {
-        const T c = G.cf;
-#pragma unroll
-        for (int m = 0; m < RPT; ++m) axpy(y[m], c, xp[m]);
-      }
-      if (fl & kPatReg) reg_lanes<1>(y, xp, odd ? G.co[0] : G.ce[0], odd ? G.ce[0] : G.co[0]);
-      if (fl & (kPatReg << 1)) reg_lanes<2>(y, xp, odd ? G.co[1] : G.ce[1], odd ? G.ce[1] : G.co[1]);
-      if (fl & (kPatReg << 2)) reg_lanes<4>(y, xp, odd ? G.co[2] : G.ce[2], odd ? G.ce[2] : G.co[2]);
-    }
-    // terms of the row-group spins alone
-    if constexpr (UNI) {
-      int t = 0;
-      for (; t + 1 < tt.n_own; t += 2)
-        rows_fma2<kStep>(y, own + (rgoff ^ (int)lanet[t].off), lanet[t].co, own + (rgoff ^ (int)lanet[t + 1].off),
-                         lanet[t + 1].co);
-      if (t < tt.n_own) rows_fma<kStep>(y, own + (rgoff ^ (int)lanet[t].off), lanet[t].co);
-    } else {
-      for (int t = 0; t < tt.n_own; ++t) {
-        const LaneS<T> d = lanet[t];
-        const T c = ((act_lane >> t) & 1u) ? d.co : d.ce;
-        // where the coefficient differs across the warp's lanes they all run the term
-        if (__any_sync(0xffffffffu, in_use(c))) rows_fma<kStep>(y, own + (rgoff ^ (int)d.off), c);
-      }
-    }
+    own_terms<UNI, RG, kStep>(y, xo, own, rgoff, tt, s_reg, grp, lanet, act_lane, act_grp);
     release();
     // Partner tiles, in the producer's order: opposite-spin pairs, single-spin patterns, the
     // flat ones in use.
-    auto single = [&](const PatS<T>& A) {  // one high spin: its field and its hops
-      const uint32_t hs = (ut & A.high) != 0u, fl = A.flags;
-      if (fl & (kPatField | (kPatReg * 7u))) {
-        T xp[RPT][VW];
-        load_rows<kStep>(xp, sp + rgoff);
-        if (fl & kPatField) {
-          const T c = A.cf;
-#pragma unroll
-          for (int m = 0; m < RPT; ++m) axpy(y[m], c, xp[m]);
-        }
-        if (fl & kPatReg) reg_uniform<1>(y, xp, hs ? A.co[0] : A.ce[0], hs ? A.ce[0] : A.co[0]);
-        if (fl & (kPatReg << 1)) reg_uniform<2>(y, xp, hs ? A.co[1] : A.ce[1], hs ? A.ce[1] : A.co[1]);
-        if (fl & (kPatReg << 2)) reg_uniform<4>(y, xp, hs ? A.co[2] : A.ce[2], hs ? A.ce[2] : A.co[2]);
-      }
-      for (int t = A.start; t < A.end; ++t) {
-        const LaneS<T> d = lanet[t];
-        const bool odd = (((uint32_t)rg & d.low) != 0u) != (hs != 0u);
-        const T c = UNI || odd ? d.co : d.ce;
-        if (UNI || __any_sync(0xffffffffu, in_use(c))) rows_fma<kStep>(y, sp + (rgoff ^ (int)d.off), c);
-      }
+    auto single = [&](const PatS<T>& A) {
+      single_terms<UNI, kStep>(y, sp, rgoff, rg, A, (ut & A.high) != 0u, lanet);
     };
     if constexpr (UNI) {
       for (int st = 0; st < n_st;) {
@@ -1168,25 +1216,7 @@ __global__ void __launch_bounds__(kTiledThreads, 1) k_spmm_tiled(Layout L, SpmmA
           break;
         }
         const PatS<T>& B = pat[stage[at].what];
-        const uint32_t fl = A.flags;
-        if (fl & (kPatReg * 7u)) {
-          T xp[RPT][VW];
-          load_rows<kStep>(xp, sp + rgoff);
-          if (fl & kPatReg) reg_half<1, 1>(y, xp, A.co[0]);
-          if (fl & (kPatReg << 1)) reg_half<2, 1>(y, xp, A.co[1]);
-          if (fl & (kPatReg << 2)) reg_half<4, 1>(y, xp, A.co[2]);
-          load_rows<kStep>(xp, sb + rgoff);
-          if (fl & kPatReg) reg_half<1, 0>(y, xp, B.co[0]);
-          if (fl & (kPatReg << 1)) reg_half<2, 0>(y, xp, B.co[1]);
-          if (fl & (kPatReg << 2)) reg_half<4, 0>(y, xp, B.co[2]);
-        }
-        const int n = A.end - A.start;
-        const LaneS<T>* const la = lanet + A.start;
-        const LaneS<T>* const lb = lanet + B.start;
-        for (int t = 0; t < n; ++t) {
-          const bool up = ((uint32_t)rg & la[t].low) != 0u;
-          rows_fma<kStep>(y, (up ? sp : sb) + (rgoff ^ (int)la[t].off), up ? la[t].co : lb[t].co);
-        }
+        pair_terms<kStep>(y, sp, sb, rgoff, rg, A, B, lanet);
         release2();
         st += 2;
       }
@@ -2034,16 +2064,11 @@ __global__ void k_small_a(Layout L, const double* partials, const double* mz, do
   small_a_group<DS>(L, partials, mz, a_out, cw_out, flags, blockIdx.x);
 }
 
-// After the orthogonalisation, for group l (every thread of the block calls it): the
-// Cholesky QR with deflation -> B_j, M_{j+1}, Cp_{j+1}.
+// One group's Cholesky QR with deflation from the Gram `tot`: B_j, M_{j+1}, Cp_{j+1} = -M_j
+// B_j^T. Returns whether a column was dropped.
 template <int DS>
-__device__ void small_b_group(const Layout& L, const double* partials, const double* mz_j, double* b_out,
-                              double* mz_next, double* cp_next, double thr_abs_sq, double thr_rel_sq,
-                              int n_real, uint32_t* flags, int l) {
-  constexpr int NV = DS * DS;
-  __shared__ double tot[NV];
-  reduce_group<NV>(L, partials, tot, l);
-  if (threadIdx.x != 0) return;
+__device__ bool qr_group(const double* tot, const double* Mj, double thr_abs_sq, double thr_rel_sq, double* b_out,
+                         double* mz_next, double* cp_next, bool& finite) {
   double G[DS][DS], R[DS][DS], Ri[DS][DS];
   bool kept[DS];
   for (int i = 0; i < DS; ++i)
@@ -2054,7 +2079,8 @@ __device__ void small_b_group(const Layout& L, const double* partials, const dou
     }
   // Cholesky G = R^T R column by column, dropping numerically dependent columns
   // (Gram-Schmidt in the G inner product; same rule as a column-wise QR).
-  bool dropped = false, finite = true;
+  bool dropped = false;
+  finite = true;
   for (int c = 0; c < DS; ++c) {
     for (int k = 0; k < c; ++k) {
       if (!kept[k]) continue;
@@ -2088,15 +2114,30 @@ __device__ void small_b_group(const Layout& L, const double* partials, const dou
       Ri[r][c] = -s / R[r][r];
     }
   }
-  const double* Mj = mz_j + (size_t)l * NV;
   for (int i = 0; i < DS; ++i)
     for (int j = 0; j < DS; ++j) {
-      b_out[(size_t)l * NV + i * DS + j] = R[i][j];
-      mz_next[(size_t)l * NV + i * DS + j] = Ri[i][j];
+      b_out[i * DS + j] = R[i][j];
+      mz_next[i * DS + j] = Ri[i][j];
       double s = 0.0;
       for (int c = 0; c < DS; ++c) s += Mj[i * DS + c] * R[j][c];
-      cp_next[(size_t)l * NV + i * DS + j] = -s;
+      cp_next[i * DS + j] = -s;
     }
+  return dropped;
+}
+
+// After the orthogonalisation, for group l (every thread of the block calls it): the
+// Cholesky QR with deflation -> B_j, M_{j+1}, Cp_{j+1}.
+template <int DS>
+__device__ void small_b_group(const Layout& L, const double* partials, const double* mz_j, double* b_out,
+                              double* mz_next, double* cp_next, double thr_abs_sq, double thr_rel_sq,
+                              int n_real, uint32_t* flags, int l) {
+  constexpr int NV = DS * DS;
+  __shared__ double tot[NV];
+  reduce_group<NV>(L, partials, tot, l);
+  if (threadIdx.x != 0) return;
+  const size_t o = (size_t)l * NV;
+  bool finite;
+  const bool dropped = qr_group<DS>(tot, mz_j + o, thr_abs_sq, thr_rel_sq, b_out + o, mz_next + o, cp_next + o, finite);
   if (dropped && l < n_real) atomicOr(flags, (uint32_t)RDM_FLAG_DEFLATED);
   if (!finite) atomicOr(flags, kFlagNonFinite);
 }
@@ -2288,6 +2329,306 @@ __global__ void __launch_bounds__(kThreads) k_pass1_local(PackedPlan pp) {
       __syncthreads();
     }
   }
+}
+
+// ---------------------------------------------------------------- first pass in a cluster
+//
+// The whole first pass of one slice (float32, 2^kTileBits states per block) in one
+// thread-block cluster: block `rank` keeps tile `rank` of W_j, and of W_{j-1}, in its shared
+// memory for all k steps, reads partner tiles from the other blocks' shared memory, and the
+// partial sums of A_j and of the QR Gram are exchanged the same way. A slice's recurrences
+// read nothing of other slices, so no step needs more than two cluster barriers; every block
+// of a cluster passes the same ones (k is the slice's), so each of them ends. Stored bases
+// are written to global memory as they are formed. Every row's arithmetic is the tiled
+// SpMM's and the orthogonalisation's, in their order (pass 2 recomputes the same bits).
+//
+// Bound by latency and the terms' shared-memory loads; two blocks per SM (at 128 registers,
+// some spilled) hide more of it than one. It replaces, for batches, the untiled units of
+// k_pass1_packed on items of 2^10 .. 2^14 states, which read every partner row from L2: the
+// first passes of 48 small solves (N 8-14) take 44 instead of 87 ms.
+constexpr int kClusterThreads = kConsumerWarps * 32;
+constexpr int kClusterMaxLog = 4;  // up to 16 blocks (N = 14)
+
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release;\nbarrier.cluster.wait.acquire;\n" ::: "memory");
+}
+// The same shared-memory address in block `rank` of the cluster.
+template <typename P>
+__device__ __forceinline__ const P* peer(const P* p, uint32_t rank) {
+  uint64_t r;
+  asm volatile("mapa.u64 %0, %1, %2;" : "=l"(r) : "l"(reinterpret_cast<uint64_t>(p)), "r"(rank));
+  return reinterpret_cast<const P*>(r);
+}
+
+__host__ __device__ inline size_t cluster_smem_bytes(const TiledTerms& tt) {
+  return 2 * (size_t)kTileBytes + 8 * 32 * sizeof(double) + (size_t)kConsumerWarps * 2 * 16 * sizeof(double) +
+         (size_t)tt.n_part * sizeof(PatS<float>) + (size_t)tt.n_grp * sizeof(GrpS<float>) +
+         (size_t)tt.n_lane * sizeof(LaneS<float>) +
+         sizeof(float) * (16 + 4 * 32 + kTileRows + (size_t)tile_diag_stride(tt.dg.n_entries, 4)) + 64;
+}
+
+template <int DS>
+__global__ void __launch_bounds__(kClusterThreads, 2) k_pass1_cluster(PackedPlan pp, int c_log) {
+  using T = float;
+  constexpr int VW = 4, LPR = 2, BS = VW * LPR, RG = kClusterThreads / LPR, RPT = kTileRows / RG;
+  constexpr int kStep = RG * BS, kTile = kTileRows * BS;
+  constexpr int NG = VW / DS, NVG = DS * DS, NV = NG * NVG;
+  constexpr int GS = LPR * NG, GV = GS * NVG;  // groups of the slice and their values
+  const uint32_t rank = blockIdx.x & ((1u << c_log) - 1u), peers = 1u << c_log;
+  const int u = blockIdx.x >> c_log;
+  const int item = packed_item_of(pp.pre_slices, pp.n_items, u);
+  const PackedItem& it = pp.items[item];
+  const int slice = u - pp.pre_slices[item];
+  const TiledTerms& tt = it.sa.tiled;
+  extern __shared__ __align__(128) unsigned char smem_c[];
+  T* const buf = reinterpret_cast<T*>(smem_c);
+  double* const sM = reinterpret_cast<double*>(buf + 2 * kTile);  // M_j of the slice's groups
+  double* const sMn = sM + 32;
+  double* const sCp = sM + 64;
+  double* const sTot = sM + 96;
+  double* const sA = sM + 128;
+  double* const sR = sM + 160;
+  double* const part_a = sM + 192;  // this block's sums of W_j^T Z ...
+  double* const part_b = sM + 224;  // ... and of W_{j+1}^T W_{j+1}
+  double* const red = sM + 256;     // [warp][lane][NV]
+  PatS<T>* const pat = reinterpret_cast<PatS<T>*>(red + kConsumerWarps * 2 * 16);
+  GrpS<T>* const grp = reinterpret_cast<GrpS<T>*>(pat + tt.n_part);
+  LaneS<T>* const lanet = reinterpret_cast<LaneS<T>*>(grp + tt.n_grp);
+  T* const s_reg = reinterpret_cast<T*>(lanet + tt.n_lane);
+  T* const s_mz = s_reg + 16;
+  T* const s_cp = s_mz + 32;
+  T* const s_cw = s_cp + 32;
+  T* const s_low = s_cw + 64;
+  T* const s_hk = s_low + kTileRows;
+
+  load_tables<BS>(tt, pat, grp, lanet, s_reg, s_low);
+  const int hstride = tile_diag_stride(tt.dg.n_entries, (int)sizeof(T));
+  for (int i = threadIdx.x; i < hstride; i += kClusterThreads)
+    s_hk[i] = reinterpret_cast<const T*>(it.sa.tile_k)[(size_t)rank * hstride + i];
+  const int lane = threadIdx.x % LPR, rg = threadIdx.x / LPR, warp = threadIdx.x >> 5;
+  const int rgoff = rg * BS + lane * VW;
+  const size_t bb = it.L.block_bytes(), cs = (size_t)it.L.n_groups() * NVG, go = (size_t)slice * GV;
+  // this thread's first row in block 0 of the basis
+  const size_t row_b = ((size_t)slice * it.L.D * BS + (size_t)rank * kTile + rgoff) * sizeof(T);
+  T xo[RPT][VW];
+  load_rows<kStep>(xo, reinterpret_cast<const T*>(it.blk + row_b));
+#pragma unroll
+  for (int m = 0; m < RPT; ++m) VecIO<T, VW>::st(buf + rgoff + m * kStep, xo[m]);
+  if (threadIdx.x < GV) {
+    sM[threadIdx.x] = it.coef[cs + go + threadIdx.x];
+    s_mz[threadIdx.x] = (T)sM[threadIdx.x];
+    s_cp[threadIdx.x] = (T)0;
+  }
+  __syncthreads();
+  uint32_t act_lane = 0u, act_grp = 0u;
+  for (int t = 0; t < tt.n_own; ++t) act_lane |= (uint32_t)(__popc((uint32_t)rg & lanet[t].low) & 1) << t;
+  for (int t = 0; t < tt.n_grp; ++t) act_grp |= (uint32_t)(((uint32_t)rg & grp[t].low) != 0u) << t;
+  // patterns whose high spin is up (bit p) in this block's tile
+  uint32_t up_pairs = 0u;
+  for (int p = 0; p < tt.n_pair; ++p) up_pairs |= (uint32_t)((rank & pat[p].high) != 0u) << p;
+  cluster_sync();
+
+  // The block's sums of NV values per thread over the threads of a lane: out[lane][NV].
+  auto block_sums = [&](const T* vals, double* out) {
+#pragma unroll
+    for (int e = 0; e < NV; ++e) {
+      T x = vals[e];
+#pragma unroll
+      for (int o = LPR; o < 32; o <<= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+      if ((threadIdx.x & 31) < LPR) red[(warp * LPR + lane) * 16 + e] = (double)x;
+    }
+    __syncthreads();
+    if (threadIdx.x < GV) {
+      const int ln = threadIdx.x / NV, e = threadIdx.x % NV;
+      double sum = 0.0;
+      for (int w = 0; w < kConsumerWarps; ++w) sum += red[(w * LPR + ln) * 16 + e];
+      out[threadIdx.x] = sum;
+    }
+  };
+  // The cluster's sums of part (after a cluster barrier), the blocks in order.
+  auto cluster_sums = [&](const double* part) {
+    if (threadIdx.x < GV) {
+      double sum = 0.0;
+      for (uint32_t r = 0; r < peers; ++r) sum += peer(part, r)[threadIdx.x];
+      sTot[threadIdx.x] = sum;
+    }
+    __syncthreads();
+  };
+
+  for (int j = 1; j <= it.k; ++j) {
+    const T* const cur = buf + ((j - 1) & 1) * kTile;  // W_j
+    T* const oth = buf + (j & 1) * kTile;              // W_{j-1}, then W_{j+1}
+    T y[RPT][VW];
+    {
+      T dg[RPT];
+      tile_diagonal<T, RPT, RG>(dg, s_low, s_hk, rg, tt.dg);
+#pragma unroll
+      for (int m = 0; m < RPT; ++m)
+#pragma unroll
+        for (int v = 0; v < VW; ++v) y[m][v] = dg[m] * xo[m][v];
+    }
+    own_terms<false, RG, kStep>(y, xo, cur, rgoff, tt, s_reg, grp, lanet, act_lane, act_grp);
+    // partner tiles in the tiled SpMM's order
+    uint32_t om = up_pairs, zm = ~up_pairs & (uint32_t)((1u << tt.n_pair) - 1u);
+    for (int joint = min(__popc(zm), __popc(om)); zm | om; --joint) {
+      if (joint > 0) {
+        const int z = __ffs((int)zm) - 1, o = __ffs((int)om) - 1;
+        zm &= zm - 1u;
+        om &= om - 1u;
+        pair_terms<kStep>(y, peer(cur, rank ^ pat[z].high), peer(cur, rank ^ pat[o].high), rgoff, rg, pat[z], pat[o],
+                          lanet);
+      } else {
+        const int p = __ffs((int)(zm | om)) - 1;
+        zm &= ~(1u << p);
+        om &= ~(1u << p);
+        single_terms<false, kStep>(y, peer(cur, rank ^ pat[p].high), rgoff, rg, pat[p], (rank & pat[p].high) != 0u, lanet);
+      }
+    }
+    for (int p = tt.n_pair; p < tt.n_pair + tt.n_single; ++p)
+      single_terms<false, kStep>(y, peer(cur, rank ^ pat[p].high), rgoff, rg, pat[p], (rank & pat[p].high) != 0u, lanet);
+    for (int p = tt.n_pair + tt.n_single; p < tt.n_part; ++p) {
+      const T c = (__popc(rank & pat[p].high) & 1) ? pat[p].co[0] : pat[p].ce[0];
+      if (in_use(c)) rows_fma<kStep>(y, peer(cur, rank ^ pat[p].high) + rgoff, c);
+    }
+    // Z = (H W_j) M_j + W_{j-1} Cp_j into y, and the sums of W_j^T Z
+    T vals[NV];
+#pragma unroll
+    for (int e = 0; e < NV; ++e) vals[e] = (T)0;
+    {
+      T mz[NV], cp[NV];
+#pragma unroll
+      for (int e = 0; e < NV; ++e) {
+        mz[e] = s_mz[lane * NV + e];
+        cp[e] = s_cp[lane * NV + e];
+      }
+#pragma unroll
+      for (int m = 0; m < RPT; ++m) {
+        T z[VW];
+#pragma unroll
+        for (int g = 0; g < NG; ++g)
+#pragma unroll
+          for (int c = 0; c < DS; ++c) {
+            T t = (T)0;
+#pragma unroll
+            for (int i = 0; i <= c; ++i) t = fma(y[m][g * DS + i], mz[g * NVG + i * DS + c], t);
+            z[g * DS + c] = t;
+          }
+        if (j > 1) {
+          T xp[VW];
+          VecIO<T, VW>::ld_rw(xp, oth + rgoff + m * kStep);
+#pragma unroll
+          for (int g = 0; g < NG; ++g)
+#pragma unroll
+            for (int c = 0; c < DS; ++c) {
+              T t = z[g * DS + c];
+#pragma unroll
+              for (int i = 0; i < DS; ++i) t = fma(xp[g * DS + i], cp[g * NVG + i * DS + c], t);
+              z[g * DS + c] = t;
+            }
+        }
+#pragma unroll
+        for (int g = 0; g < NG; ++g)
+#pragma unroll
+          for (int i = 0; i < DS; ++i)
+#pragma unroll
+            for (int c = 0; c < DS; ++c)
+              vals[g * NVG + i * DS + c] = fma(xo[m][g * DS + i], z[g * DS + c], vals[g * NVG + i * DS + c]);
+#pragma unroll
+        for (int v = 0; v < VW; ++v) y[m][v] = z[v];
+      }
+    }
+    block_sums(vals, part_a);
+    cluster_sync();
+    cluster_sums(part_a);
+    // A_j and Cw_j (small_a_group): thread e of the slice's values
+    const int e = threadIdx.x, g = e / NVG, r = e % NVG / DS, c = e % DS;
+    if (e < GV) {
+      double p1 = 0.0, p2 = 0.0;  // (Q_j^T Z)[r][c] and [c][r]
+      for (int i = 0; i < DS; ++i) {
+        p1 += sM[g * NVG + i * DS + r] * sTot[g * NVG + i * DS + c];
+        p2 += sM[g * NVG + i * DS + c] * sTot[g * NVG + i * DS + r];
+      }
+      sA[e] = 0.5 * (p1 + p2);
+    }
+    __syncthreads();
+    if (e < GV) {
+      double cw = 0.0;
+      for (int i = 0; i < DS; ++i) cw += sM[g * NVG + r * DS + i] * sA[g * NVG + i * DS + c];
+      s_cw[e] = (T)-cw;
+      if (rank == 0) {
+        it.ta[(size_t)(j - 1) * cs + go + e] = sA[e];
+        it.coef[(size_t)2 * (it.k + 2) * cs + (size_t)j * cs + go + e] = -cw;
+        if (!isfinite(sA[e])) atomicOr(it.flags, kFlagNonFinite);
+      }
+    }
+    __syncthreads();
+    // W_{j+1} = Z + W_j Cw_j, its sums, its rows kept
+    {
+      T cw[NV];
+#pragma unroll
+      for (int q = 0; q < NV; ++q) {
+        cw[q] = s_cw[lane * NV + q];
+        vals[q] = (T)0;
+      }
+      T* const out = reinterpret_cast<T*>(it.blk + (size_t)j * bb + row_b);
+#pragma unroll
+      for (int m = 0; m < RPT; ++m) {
+#pragma unroll
+        for (int q = 0; q < NG; ++q)
+#pragma unroll
+          for (int cc = 0; cc < DS; ++cc) {
+            T t = y[m][q * DS + cc];
+#pragma unroll
+            for (int i = 0; i < DS; ++i) t = fma(xo[m][q * DS + i], cw[q * NVG + i * DS + cc], t);
+            y[m][q * DS + cc] = t;
+          }
+#pragma unroll
+        for (int q = 0; q < NG; ++q)
+#pragma unroll
+          for (int i = 0; i < DS; ++i)
+#pragma unroll
+            for (int cc = i; cc < DS; ++cc)
+              vals[q * NVG + i * DS + cc] = fma(y[m][q * DS + i], y[m][q * DS + cc], vals[q * NVG + i * DS + cc]);
+        VecIO<T, VW>::st(oth + rgoff + m * kStep, y[m]);
+        VecIO<T, VW>::st_cs(out + m * kStep, y[m]);
+#pragma unroll
+        for (int v = 0; v < VW; ++v) xo[m][v] = y[m][v];
+      }
+#pragma unroll
+      for (int q = 0; q < NG; ++q)
+#pragma unroll
+        for (int i = 0; i < DS; ++i)
+#pragma unroll
+          for (int cc = 0; cc < i; ++cc) vals[q * NVG + i * DS + cc] = vals[q * NVG + cc * DS + i];
+    }
+    block_sums(vals, part_b);
+    cluster_sync();  // W_{j+1} and part_b of every block are there
+    cluster_sums(part_b);
+    // B_j, M_{j+1}, Cp_{j+1} (small_b_group): one thread per group
+    if (threadIdx.x < GS) {
+      const int o = threadIdx.x * NVG;
+      bool finite;
+      const bool dropped =
+          qr_group<DS>(sTot + o, sM + o, it.thr_abs_sq, it.thr_rel_sq, sR + o, sMn + o, sCp + o, finite);
+      if (rank == 0) {
+        if (dropped && slice * GS + (int)threadIdx.x < it.n_rec) atomicOr(it.flags, (uint32_t)RDM_FLAG_DEFLATED);
+        if (!finite) atomicOr(it.flags, kFlagNonFinite);
+      }
+    }
+    __syncthreads();
+    if (e < GV) {
+      sM[e] = sMn[e];
+      s_mz[e] = (T)sMn[e];
+      s_cp[e] = (T)sCp[e];
+      if (rank == 0) {
+        it.tb[(size_t)(j - 1) * cs + go + e] = sR[e];
+        it.coef[(size_t)(j + 1) * cs + go + e] = sMn[e];
+        it.coef[(size_t)(it.k + 2) * cs + (size_t)(j + 1) * cs + go + e] = sCp[e];
+      }
+    }
+    __syncthreads();
+  }
+  cluster_sync();  // no block leaves while another may still read its shared memory
 }
 
 inline dim3 grid_of(const Layout& L) { return dim3((unsigned)L.gridx, (unsigned)L.n_slices); }
@@ -2580,6 +2921,40 @@ cudaError_t launch_pass1_local(int precision, int ds, const PackedPlan& pp, int 
   void* args[] = {&arg};
   return cudaLaunchKernel(fn, dim3((unsigned)grid), dim3(kThreads), args, smem, st);
 }
+
+bool pass1_cluster_fits(const Layout& L, const TiledTerms& tt) {
+  return L.precision == RDM_FP32 && layout_tiled(L) && tt.ready && L.n_bits - kTileBits <= kClusterMaxLog &&
+         cluster_smem_bytes(tt) <= (size_t)200 * 1024;
+}
+
+cudaError_t launch_pass1_cluster(int ds, const PackedPlan& pp, int c_log, int n_slices, size_t smem, cudaStream_t st) {
+  if (c_log < 0 || c_log > kClusterMaxLog) return cudaErrorInvalidValue;
+  auto go = [&](auto d) -> cudaError_t {
+    constexpr int DS = decltype(d)::value;
+    const void* fn = reinterpret_cast<const void*>(k_pass1_cluster<DS>);
+    cudaError_t e = opt_in_smem(fn);
+    // (16 blocks exceed the portable cluster size)
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)n_slices << c_log);
+    cfg.blockDim = dim3(kClusterThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = 1u << c_log;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k_pass1_cluster<DS>, pp, c_log);
+  };
+  if (ds == 1) return go(std::integral_constant<int, 1>{});
+  if (ds == 2) return go(std::integral_constant<int, 2>{});
+  return go(std::integral_constant<int, 4>{});
+}
+
+size_t pass1_cluster_smem(const TiledTerms& tt) { return cluster_smem_bytes(tt); }
 
 cudaError_t launch_pass1_packed(int precision, int ds, const PackedPlan& pp, int grid, size_t smem,
                                 cudaStream_t st) {

@@ -165,3 +165,35 @@ def test_batch_launch_forms_are_bit_identical(lib):
         assert e.value.status == lib.EINVAL
     finally:
         ctx.close()
+
+
+@pytest.mark.parametrize("n", [10, 11, 12, 13, 14])
+@pytest.mark.parametrize("n_sys", [0, 1, 2])
+def test_batch_first_passes_in_clusters(lib, n, n_sys):
+    """float32 items of 2^10..2^14 states run their first pass in one thread-block cluster per
+    slice (1 to 16 blocks): T's coefficients against the untiled units (form 1) over the
+    first steps, within the float32 rounding of six steps; the whole estimate within the
+    float32 contract; alone, in the mix and in another order bit for bit the same."""
+    specs = [W.long_range_xxz(n, n_sys, 1.0, 0.8, 0.3, 0.7), W.random_model(n, n_sys, n),
+             W.long_range_tfim(n, n_sys, 1.5, 0.9), W.xxz_chain(n, n_sys, 1.0, 0.5, 0.1)]
+    ctx = lib.Context(0)
+    try:
+        jobs = [dict(ham=lib.Hamiltonian(ctx, s), betas=W.beta_grid(9, 0.1, 4.0), n_v=v, k=k, seed=40 + v,
+                     precision="fp32", dist="gauss") for s, v, k in zip(specs, (1, 7, 16, 5), (18, 6, 25, 12))]
+        mix = ctx.estimate_batch(jobs, full=True)
+        rev = ctx.estimate_batch(jobs[::-1], full=True)[::-1]
+        ctx.set_packed_form(1)
+        plain = ctx.estimate_batch(jobs, full=True)
+        ctx.set_packed_form(0)
+        for jb, a, b, p in zip(jobs, mix, rev, plain):
+            alone = ctx.estimate_batch([jb], full=True)[0]
+            for key in ("rho", "lnZ", "gram_l", "t_a", "t_b"):
+                np.testing.assert_array_equal(a[key], b[key])
+                np.testing.assert_array_equal(a[key], alone[key])
+            bound = jb["ham"].info()["norm_bound"]
+            for key in ("t_a", "t_b"):
+                np.testing.assert_allclose(a[key][:, :6], p[key][:, :6], atol=2e-5 * bound, rtol=0)
+            np.testing.assert_allclose(a["rho"], p["rho"], atol=1e-4, rtol=0)
+            np.testing.assert_allclose(a["rho"], a["rho_quad"], atol=1e-4, rtol=0)
+    finally:
+        ctx.close()
