@@ -65,35 +65,40 @@ __device__ __forceinline__ int job_of(const int* pre, int n, int g) {
 
 // Eigenvalues of T - sigma I below zero, in arithmetic R (block LDL^T with no pivoting
 // inside the d_s x d_s blocks; a pivot smaller than pivmin counts as negative and is
-// replaced by -pivmin).
+// replaced by -pivmin). Only lower triangles are formed: D_j is symmetric, and B_j is upper
+// triangular (the Cholesky factor, exact zeros below), so X = L^{-1} B_j^T is lower
+// triangular. One warp works through the k blocks in a row, bound by the float64 pipe's
+// latency and rate: 76 operations and d_s divisions a block instead of 190 (d_s = 4; 45 steps
+// 2.24 -> 1.34 ms).
 template <int DS, typename R>
 __device__ int count_below(int k, int ng, int g, const double* ta, const double* tb, R sigma, R pivmin) {
   constexpr int NV = DS * DS;
-  R D[DS][DS];
+  R D[DS][DS];  // lower triangle
 #pragma unroll
   for (int a = 0; a < DS; ++a)
 #pragma unroll
-    for (int b = 0; b < DS; ++b) D[a][b] = (R)ta[(size_t)g * NV + a * DS + b] - (a == b ? sigma : (R)0);
+    for (int b = 0; b <= a; ++b) D[a][b] = (R)ta[(size_t)g * NV + a * DS + b] - (a == b ? sigma : (R)0);
   int cnt = 0;
   for (int j = 0;; ++j) {
     R L[DS][DS], d[DS], id[DS];
 #pragma unroll
     for (int i = 0; i < DS; ++i) {
+      R w[DS];  // L[i][m] d[m]
       R di = D[i][i];
 #pragma unroll
-      for (int m = 0; m < DS; ++m)
-        if (m < i) di -= L[i][m] * L[i][m] * d[m];
+      for (int m = 0; m < i; ++m) {
+        w[m] = L[i][m] * d[m];
+        di -= L[i][m] * w[m];
+      }
       if (!(fabs(di) >= pivmin)) di = -pivmin;  // also catches NaN
       if (di < (R)0) ++cnt;
       d[i] = di;
       id[i] = (R)1 / di;
 #pragma unroll
-      for (int r = 0; r < DS; ++r) {
-        if (r <= i) continue;
+      for (int r = i + 1; r < DS; ++r) {
         R x = D[r][i];
 #pragma unroll
-        for (int m = 0; m < DS; ++m)
-          if (m < i) x -= L[r][m] * L[i][m] * d[m];
+        for (int m = 0; m < i; ++m) x -= L[r][m] * w[m];
         L[r][i] = x * id[i];
       }
     }
@@ -101,26 +106,26 @@ __device__ int count_below(int k, int ng, int g, const double* ta, const double*
     // D_{j+1} = A_{j+1} - sigma I - B_j D_j^{-1} B_j^T; with X = L^{-1} B_j^T,
     // B_j D_j^{-1} B_j^T = X^T diag(1/d) X.
     const double* B = tb + ((size_t)j * ng + g) * NV;
-    R X[DS][DS];
+    R X[DS][DS], Y[DS][DS];
 #pragma unroll
     for (int c = 0; c < DS; ++c)      // column c of B_j^T = row c of B_j
 #pragma unroll
-      for (int i = 0; i < DS; ++i) {  // forward substitution with unit lower L
+      for (int i = c; i < DS; ++i) {  // forward substitution with unit lower L
         R x = (R)blk(B, DS, c, i);
 #pragma unroll
-        for (int m = 0; m < DS; ++m)
-          if (m < i) x -= L[i][m] * X[m][c];
+        for (int m = c; m < i; ++m) x -= L[i][m] * X[m][c];
         X[i][c] = x;
+        Y[i][c] = x * id[i];
       }
     const double* A = ta + ((size_t)(j + 1) * ng + g) * NV;
 #pragma unroll
     for (int a = 0; a < DS; ++a)
 #pragma unroll
-      for (int b = 0; b < DS; ++b) {
-        R s = (R)0;
+      for (int b = 0; b <= a; ++b) {
+        R s = (R)blk(A, DS, a, b) - (a == b ? sigma : (R)0);
 #pragma unroll
-        for (int i = 0; i < DS; ++i) s += X[i][a] * X[i][b] * id[i];
-        D[a][b] = (R)blk(A, DS, a, b) - (a == b ? sigma : (R)0) - s;
+        for (int i = a; i < DS; ++i) s -= X[i][a] * Y[i][b];
+        D[a][b] = s;
       }
   }
   return cnt;
@@ -324,13 +329,21 @@ __global__ void __launch_bounds__(kChebThreads) k_cheb_combine(const DenseJob* j
   const int n = J.k * DS, ne = n * DS;
   const double lo = J.lohi[2 * g], top = J.lohi[2 * g + 1];
   const double width = top - lo > 0.0 ? top - lo : 1.0;
-  const int m = cheb_degree(J.beta_max * width / 4.0, vstride);
+  // Every beta has its own degree (the one its coefficients reach 1e-17 at): the sums are
+  // bound by the float64 pipe, and on a geometric grid of 0.1 to 10 the average degree is
+  // 0.4 of the largest.
+  __shared__ int deg[kCombineBetas];
   if ((int)threadIdx.x < nb) {
     double* al = sa + (size_t)threadIdx.x * vstride;
-    scaled_bessel_i(J.betas[b0 + threadIdx.x] * width / 4.0, m, al);
-    for (int i = 1; i <= m; ++i) al[i] *= (i & 1) ? -2.0 : 2.0;
+    const double omega = J.betas[b0 + threadIdx.x] * width / 4.0;
+    const int mb = cheb_degree(omega, vstride);
+    scaled_bessel_i(omega, mb, al);
+    for (int i = 1; i <= mb; ++i) al[i] *= (i & 1) ? -2.0 : 2.0;
+    deg[threadIdx.x] = mb;
   }
   __syncthreads();
+  int m = 0;
+  for (int b = 0; b < nb; ++b) m = max(m, deg[b]);
   const double* Vg = J.V + (size_t)g * vstride * ne;
   for (int e = threadIdx.x; e < ne; e += blockDim.x) {
     double acc[kCombineBetas];
@@ -340,7 +353,7 @@ __global__ void __launch_bounds__(kChebThreads) k_cheb_combine(const DenseJob* j
       const double v = Vg[(size_t)i * ne + e];
 #pragma unroll
       for (int b = 0; b < kCombineBetas; ++b)
-        if (b < nb) acc[b] = fma(sa[(size_t)b * vstride + i], v, acc[b]);
+        if (b < nb && i <= deg[b]) acc[b] = fma(sa[(size_t)b * vstride + i], v, acc[b]);
     }
 #pragma unroll
     for (int b = 0; b < kCombineBetas; ++b)
