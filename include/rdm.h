@@ -313,20 +313,25 @@ typedef struct {
 } rdm_batch_item;
 
 /* Many estimates at once, of Hamiltonians of any sizes (the paper's independent
- * recurrences of Sec. 3.1, over several models): every item that keeps its Krylov basis
- * (k+1 blocks fit) and whose block is at most 64 MB runs its first pass (Algorithm 1's k
- * steps) in ONE persistent cooperative launch with the other such items of its
- * precision and d_s -- the SpMM, A_j, orthogonalisation and QR phases of every item,
- * separated by grid barriers; larger items run as rdm_estimate does. Each work unit of
- * that launch is one block of the plain kernels of its item, so an item's result does
- * not depend on which other items share the batch (bit-identical alone or in any mix).
- * Its launch form is chosen by an autotuner: the cooperative grid with 1, 2, 4 or 8
- * blocks per SM (as many as fit; grid barriers between the phases of a step), or one
- * block per slice of each item running all its steps with block barriers only (the
- * recurrences of a slice read nothing of other slices; no co-residency needed). The
- * first batch of each size class times the candidates and the fastest is kept on the
- * context; every form runs the same units with the same arithmetic, so the choice
- * changes no result (rdm_set_packed_form restricts it).
+ * recurrences of Sec. 3.1, over several models). How an item's first pass (Algorithm 1's k
+ * steps) runs depends on its own sizes only:
+ *   - float32 items of 2^10 .. 2^14 states that keep their Krylov basis (k+1 blocks fit) with
+ *     a block of at most 64 MB: one thread-block cluster per slice (bath vectors of one
+ *     32-byte row), all steps in the clusters' shared memory, one launch per (d_s, N) over
+ *     all such items;
+ *   - larger float32 items whose block the tiled SpMM takes, and items above 64 MB or with a
+ *     recomputed basis: as rdm_estimate does;
+ *   - the others (N < 10, float64) in ONE persistent cooperative launch with the other such
+ *     items of their precision and d_s -- the SpMM, A_j, orthogonalisation and QR phases of
+ *     every item, separated by grid barriers. Each work unit of that launch is one block of
+ *     the plain kernels of its item. Its launch form is chosen by an autotuner: the
+ *     cooperative grid with 1, 2, 4 or 8 blocks per SM (as many as fit), or one block per
+ *     slice of each item running all its steps with block barriers only. The first batch of
+ *     each size class times the candidates and the fastest is kept on the context; every
+ *     form runs the same units with the same arithmetic, so the choice changes no result.
+ * An item's result does not depend on which other items share the batch (bit-identical
+ * alone or in any mix). rdm_set_packed_form 1 and 2 put every item that fits into the
+ * packed launch (results agree with the default's within rounding).
  * Items whose workspaces do not fit the device together run in consecutive
  * sub-batches. Blocking. Returns RDM_OK when every item succeeded, else the first
  * failure (each item's own status is in items[i].status); RDM_EINVAL for a NULL
@@ -346,9 +351,11 @@ rdm_status rdm_packed_tuning(rdm_ctx* ctx, int* n_keys, uint64_t* tuning_runs);
  * the tiled kernel where it can. RDM_EINVAL for another value. */
 rdm_status rdm_set_spmm_form(rdm_ctx* ctx, int form);
 
-/* Launch forms rdm_estimate_batch's first pass may take: 0 (the default) any, chosen
- * by the autotuner; 1 only the cooperative grid; 2 only one block per slice. The
- * tuned choices of the context are cleared. RDM_EINVAL for another value. */
+/* Launch forms rdm_estimate_batch's first pass may take: 0 (the default) the rules above,
+ * the packed launch's form chosen by the autotuner; 1 only the packed launch's cooperative
+ * grid; 2 only its one block per slice (1 and 2: every stored-basis item of at most 64 MB,
+ * bit-identical to each other). The tuned choices of the context are cleared. RDM_EINVAL for
+ * another value. */
 rdm_status rdm_set_packed_form(rdm_ctx* ctx, int form);
 
 /* Y = H X for a caller-owned device block of n_cols columns stored state-major,

@@ -10,7 +10,10 @@
 //                  accumulation psi_beta += W_{j+1} E_{j+1,beta} (pass 2)
 //   k_small_a/b    per bath vector, float64: A_j, Cholesky QR with breakdown
 //                  deflation, the next step's mixing coefficients
-//   k_final_gram   the bath-traced Gram psi_l^T psi_l per bath vector
+//   k_gram_rows    psi = sum_j W_j E_j from the stored basis and its bath-traced Gram
+//                  psi_l^T psi_l per bath vector, all betas (k_final_gram: of a given psi;
+//                  k_gram_stored: the layouts k_gram_rows does not take)
+//   k_pass1_cluster / k_pass1_packed   the whole first pass of the items of a batch
 //
 // The Krylov block of every bath vector l is never normalised in memory: the
 // stored W_j relates to the orthonormal Q_j of Algorithm 1 by Q_j = W_j M_j with

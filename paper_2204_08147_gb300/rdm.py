@@ -250,8 +250,9 @@ class Context:
         _check(_lib.rdm_set_spmm_form(self.h, int(form)), "rdm_set_spmm_form")
 
     def set_packed_form(self, form: int = 0):
-        """Launch forms of estimate_batch's packed first pass: 0 autotuned (default), 1 the
-        cooperative grid only, 2 one block per slice only (same results in every form)."""
+        """Launch forms of estimate_batch's first passes: 0 chosen by each item's sizes
+        (default: clusters, own launches, or the packed launch, autotuned), 1 the packed
+        launch's cooperative grid only, 2 its one block per slice only."""
         _check(_lib.rdm_set_packed_form(self.h, int(form)), "rdm_set_packed_form")
 
     def set_bath_order(self, enable: bool = True):
