@@ -117,6 +117,66 @@ __device__ __forceinline__ unsigned group_mask(int tpr) {
   return ((1u << tpr) - 1u) << (lane & ~(unsigned)(tpr - 1));
 }
 
+// Sums held as an unevaluated pair hi + lo of floats (Knuth's two-sum): the float32 kernels'
+// long sums, off the narrow float64 pipe.
+struct Pair32 {
+  float hi = 0.0f, lo = 0.0f;
+  __device__ __forceinline__ void add(float x) {
+    const float s = __fadd_rn(hi, x), t = __fsub_rn(s, hi);
+    lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, t)), __fsub_rn(x, t)));
+    hi = s;
+  }
+  __device__ __forceinline__ void add(const Pair32& o) {
+    add(o.hi);
+    lo = __fadd_rn(lo, o.lo);
+  }
+  __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
+};
+__device__ __forceinline__ Pair32 shfl_xor(const Pair32& p, int o) {
+  Pair32 r;
+  r.hi = __shfl_xor_sync(0xffffffffu, p.hi, o);
+  r.lo = __shfl_xor_sync(0xffffffffu, p.lo, o);
+  return r;
+}
+__device__ __forceinline__ float shfl_xor(float x, int o) { return __shfl_xor_sync(0xffffffffu, x, o); }
+__device__ __forceinline__ void add_to(float& x, float y) { x += y; }
+__device__ __forceinline__ void add_to(Pair32& x, const Pair32& y) { x.add(y); }
+
+// The sums over the 16 lanes of one parity of a warp of NV (4, 8 or 16) values, a fixed tree
+// whose every level halves the values a lane still holds (NV - 1 exchanges instead of 4 NV):
+// each lane returns one, number warp_sum_index<NV>().
+template <int NV, typename P>
+__device__ __forceinline__ P warp_sum(P (&v)[NV]) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int l = 0; l < 4; ++l) {
+    const int o = 16 >> l, half = NV >> (l + 1);
+    if (half == 0) {
+      add_to(v[0], shfl_xor(v[0], o));
+      continue;
+    }
+    const bool up = (lane & o) != 0;
+#pragma unroll
+    for (int i = 0; i < NV / 2; ++i) {
+      if (i >= half) break;
+      const P keep = up ? v[i + half] : v[i], send = up ? v[i] : v[i + half];
+      v[i] = keep;
+      add_to(v[i], shfl_xor(send, o));
+    }
+  }
+  return v[0];
+}
+template <int NV>
+__device__ __forceinline__ int warp_sum_index() {
+  static_assert(NV == 4 || NV == 8 || NV == 16, "values of a 16-byte lane");
+  return (int)(threadIdx.x & 31) >> (NV == 16 ? 1 : NV == 8 ? 2 : 3);
+}
+// One of the lanes that hold the same sum (NV < 16).
+template <int NV>
+__device__ __forceinline__ bool warp_sum_writes() {
+  return ((threadIdx.x & 31) & (NV == 16 ? 0 : NV == 8 ? 2 : 6)) == 0;
+}
+
 // Fixed-order block reduction of NV values per thread into per-block float64
 // partials: partials[((slice*gridx + bx)*G_s + lane*NG + g)*NVG + v] where
 // vals[g*NVG + v] belongs to group g of the thread and lane = threadIdx.x % tpr
@@ -150,6 +210,21 @@ __device__ void block_reduce_store(const R* vals, int tpr, double* partials, int
     for (int w = 0; w < kWarps; ++w) sum += red[(w * tpr + lane) * NV + e];
     const size_t base = (slot * gs + (size_t)lane * NG) * NVG;
     partials[base + e] = sum;
+  }
+}
+
+// The block's partials (as block_reduce_store, tpr = 2) from the warps' sums: one per lane,
+// number warp_sum_index of its column chunk.
+template <int NV>
+__device__ void warp_sums_store(const Pair32& sum, double* partials, size_t slot) {
+  constexpr int kWarps = kThreads / 32;
+  __shared__ double red[kWarps][2 * NV];
+  if (warp_sum_writes<NV>()) red[threadIdx.x >> 5][(threadIdx.x & 1) * NV + warp_sum_index<NV>()] = sum.value();
+  __syncthreads();
+  if (threadIdx.x < 2 * NV) {
+    double s = 0.0;
+    for (int w = 0; w < kWarps; ++w) s += red[w][threadIdx.x];
+    partials[slot * 2 * NV + threadIdx.x] = s;
   }
 }
 
@@ -1380,6 +1455,13 @@ __global__ void __launch_bounds__(kTiledThreads, 1) k_spmm_tiled(Layout L, SpmmA
 
 // Block (bx, by) of a gx x n_slices grid of the orthogonalisation (grid-stride rows as
 // in spmm_block).
+//
+// float32 rows of two 16-byte lanes (the tiled layout): a thread's products are summed in
+// float32 over kOrthChain rows only, then over the warp and the thread's further rows as
+// pairs of floats. How many rows a thread takes follows the grid (3 of 2^16 states with 152
+// blocks a slice, 85 with 6), and a plain float32 sum over them made B_j's rounding grow with
+// the number of bath vectors (N = 19, 1300 vectors: 5e-9 to 6e-8 of B_1).
+constexpr int kOrthChain = 16;
 template <typename T, int DS, int VW, bool PASS1, bool COH = false>
 __device__ __forceinline__ void orth_block(const Layout& L, const T* __restrict__ Wg, T* __restrict__ Zg,
                                            const double* cw, double* partials, T* psi, const double* e,
@@ -1420,6 +1502,29 @@ __device__ __forceinline__ void orth_block(const Layout& L, const T* __restrict_
     }
     __syncthreads();
   }
+  // (whole blocks of rows: every thread of a warp takes part in the warp's sums)
+  const bool chains = PASS1 && sizeof(T) == 4 && tpr == 2 && (L.D & (rpb - 1)) == 0;
+  Pair32 psum;  // the warp's sum number warp_sum_index of this lane's column chunk
+  int in_chain = 0;
+  auto fold = [&]() {
+    if constexpr (PASS1 && sizeof(T) == 4) {
+      Pair32 v[NG * NVG];
+#pragma unroll
+      for (int g = 0; g < NG; ++g)
+#pragma unroll
+        for (int i = 0; i < DS; ++i)
+#pragma unroll
+          for (int j = 0; j < DS; ++j) v[g * NVG + i * DS + j].hi = j >= i ? acc[g][i][j] : acc[g][j][i];
+      psum.add(warp_sum(v));
+#pragma unroll
+      for (int g = 0; g < NG; ++g)
+#pragma unroll
+        for (int i = 0; i < DS; ++i)
+#pragma unroll
+          for (int j = 0; j < DS; ++j) acc[g][i][j] = (T)0;
+      in_chain = 0;
+    }
+  };
   for (int64_t s = (int64_t)bx * rpb + rs; s < L.D; s += (int64_t)gx * rpb) {
     T x[VW], z[VW];
     ld_vec<T, VW, COH>(x, W + (size_t)s * L.Bs);
@@ -1443,6 +1548,7 @@ __device__ __forceinline__ void orth_block(const Layout& L, const T* __restrict_
         for (int i = 0; i < DS; ++i)
 #pragma unroll
           for (int j = i; j < DS; ++j) acc[g][i][j] = fma(z[g * DS + i], z[g * DS + j], acc[g][i][j]);
+      if (chains && ++in_chain == kOrthChain) fold();
     } else {
       for (int bi = 0; bi < nb; ++bi) {
         T* P = psi + bi * bstride + soff + (size_t)s * L.Bs;
@@ -1463,6 +1569,12 @@ __device__ __forceinline__ void orth_block(const Layout& L, const T* __restrict_
     }
   }
   if (PASS1) {
+    if constexpr (sizeof(T) == 4)
+      if (chains) {
+        if (in_chain) fold();
+        warp_sums_store<NG * NVG>(psum, partials, (size_t)by * gx + bx);
+        return;
+      }
     T vals[NG * NVG];
 #pragma unroll
     for (int g = 0; g < NG; ++g)
