@@ -916,8 +916,16 @@ __device__ __forceinline__ void load_tables(const TiledTerms& tt, PatS<T>* pat, 
   for (int i = threadIdx.x; i < kTileRows; i += blockDim.x) s_low[i] = (T)tt.dg.low[i];
 }
 
-template <typename T, int DS, int MODE, bool UNI = false>
+// TILE_SUMS (float32, pass 1): the float32 sums of W_j^T Z end with each tile; the warp's go on
+// as a pair of floats. Summed on in float32 over the runs of tiles of a slice, the rounding of
+// A_j grew with them (N = 18, 100 vectors, runs of 2 tiles: 5.7e-9 to 8.7e-9 of A_1). The
+// sums of a tile also leave the accumulators' registers to the partner tiles (XXZ N = 22 and
+// 19, XY N = 16: 1% faster solves). Not for uniform terms without runs (long slices, every
+// gridDim-th tile), whose sums stay as they were: their tiles are short, and the transverse
+// field at N = 22 would take 1.5% longer.
+template <typename T, int DS, int MODE, bool UNI = false, bool TILE_SUMS = false>
 __global__ void __launch_bounds__(kTiledThreads, 1) k_spmm_tiled(Layout L, SpmmArgs a) {
+  static_assert(!TILE_SUMS || (MODE == kModePass1 && sizeof(T) == 4), "sums of the float32 first pass");
   constexpr int VW = 16 / (int)sizeof(T);
   constexpr int LPR = kTiledLanes;          // 16-byte vectors per row
   constexpr int BS = VW * LPR;              // elements per row of a slice
@@ -1140,7 +1148,9 @@ __global__ void __launch_bounds__(kTiledThreads, 1) k_spmm_tiled(Layout L, SpmmA
     return HG ? (e / VW) * DS + (int)threadIdx.x * VW + e % VW : e;
   };
 
-  T acc[NV];  // W_j^T Z sums of this lane's bath-vector groups
+  // W_j^T Z sums of this lane's bath-vector groups, of one tile (TILE_SUMS) or of the slice
+  Pair32 psum;
+  T acc[NV];
 #pragma unroll
   for (int e = 0; e < NV; ++e) acc[e] = (T)0;
   T* __restrict__ Z = nullptr;
@@ -1166,19 +1176,22 @@ __global__ void __launch_bounds__(kTiledThreads, 1) k_spmm_tiled(Layout L, SpmmA
       if (consumers_sync_or(aborted)) aborted = true;
       if (MODE == kModePass1 && !aborted) {
         if (cur >= 0) {
-          // fixed-order reduction: shuffles within a warp (in T, like the per-thread
-          // sums), then the warps in order in float64
-          T v[NV];
+          // fixed-order reduction: the sums within a warp, then the warps in order in float64
+          if constexpr (TILE_SUMS) {
+            if (warp_sum_writes<NV>()) red[(warp * LPR + lane) * 16 + warp_sum_index<NV>()] = psum.value();
+          } else {
+            T v[NV];
 #pragma unroll
-          for (int e = 0; e < NV; ++e) {
-            T x = acc[e];
+            for (int e = 0; e < NV; ++e) {
+              T x = acc[e];
 #pragma unroll
-            for (int o = LPR; o < 32; o <<= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-            v[e] = x;
-          }
-          if ((threadIdx.x & 31) < LPR) {
+              for (int o = LPR; o < 32; o <<= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+              v[e] = x;
+            }
+            if ((threadIdx.x & 31) < LPR) {
 #pragma unroll
-            for (int e = 0; e < NV; ++e) red[(warp * LPR + lane) * 16 + e] = (double)v[e];
+              for (int e = 0; e < NV; ++e) red[(warp * LPR + lane) * 16 + e] = (double)v[e];
+            }
           }
           consumers_sync_or(false);
           if (threadIdx.x < LPR) {
@@ -1207,6 +1220,7 @@ __global__ void __launch_bounds__(kTiledThreads, 1) k_spmm_tiled(Layout L, SpmmA
         s_cp[ln * 16 + e] = has_prev ? (T)a.cp[gidx] : (T)0;
       }
       consumers_sync_or(false);
+      psum = Pair32{};
 #pragma unroll
       for (int e = 0; e < NV; ++e) acc[e] = (T)0;
     }
@@ -1446,6 +1460,11 @@ __global__ void __launch_bounds__(kTiledThreads, 1) k_spmm_tiled(Layout L, SpmmA
         }
       }
       if (has_prev) release();
+      if constexpr (TILE_SUMS) {
+        psum.add(warp_sum(acc));
+#pragma unroll
+        for (int e = 0; e < NV; ++e) acc[e] = (T)0;
+      }
     }
   }
   if (aborted && threadIdx.x == 0) atomicOr(a.err, 1u);
@@ -2867,9 +2886,9 @@ static int tiled_run_log(const Layout& L) {
   return best;
 }
 
-template <typename T, int DS, int MODE, bool UNI = false>
-static cudaError_t launch_tiled(const Layout& L, const SpmmArgs& a0, cudaStream_t st) {
-  cudaError_t e = opt_in_smem(reinterpret_cast<const void*>(k_spmm_tiled<T, DS, MODE, UNI>));
+template <typename T, int DS, int MODE, bool UNI, bool TILE_SUMS>
+static cudaError_t launch_tiled_sums(const Layout& L, const SpmmArgs& a0, int run_log, cudaStream_t st) {
+  cudaError_t e = opt_in_smem(reinterpret_cast<const void*>(k_spmm_tiled<T, DS, MODE, UNI, TILE_SUMS>));
   if (e != cudaSuccess) return e;
   static int optin = 0;
   if (!optin) {
@@ -2880,16 +2899,25 @@ static cudaError_t launch_tiled(const Layout& L, const SpmmArgs& a0, cudaStream_
   }
   // Deepest ring (up to 6 slots) that fits beside this Hamiltonian's term tables.
   SpmmArgs a = a0;
+  a.run_log = run_log;
   const TiledTerms& tt = a.tiled;
   a.stages = 6;  // a multiple of kProducerWarps
   while (a.stages > kProducerWarps &&
          tiled_smem_bytes<T>(tt.n_part, tt.n_lane, tt.n_grp, tt.dg.n_entries, a.stages) > (size_t)optin)
     a.stages -= kProducerWarps;
-  a.run_log = tiled_run_log(L);
   const size_t sm = tiled_smem_bytes<T>(tt.n_part, tt.n_lane, tt.n_grp, tt.dg.n_entries, a.stages);
   if (sm > (size_t)optin) return cudaErrorInvalidValue;
-  k_spmm_tiled<T, DS, MODE, UNI><<<dim3((unsigned)spmm_tiled_grid(L), 1), kTiledThreads, sm, st>>>(L, a);
+  k_spmm_tiled<T, DS, MODE, UNI, TILE_SUMS><<<dim3((unsigned)spmm_tiled_grid(L), 1), kTiledThreads, sm, st>>>(L, a);
   return cudaGetLastError();
+}
+
+template <typename T, int DS, int MODE, bool UNI = false>
+static cudaError_t launch_tiled(const Layout& L, const SpmmArgs& a, cudaStream_t st) {
+  const int run_log = tiled_run_log(L);
+  constexpr bool kSums = MODE == kModePass1 && sizeof(T) == 4;
+  if constexpr (kSums && UNI)
+    if (run_log == 0) return launch_tiled_sums<T, DS, MODE, UNI, false>(L, a, run_log, st);
+  return launch_tiled_sums<T, DS, MODE, UNI, kSums>(L, a, run_log, st);
 }
 
 cudaError_t launch_spmm(const Layout& L, int mode, const SpmmArgs& a, cudaStream_t st) {
