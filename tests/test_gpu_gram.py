@@ -60,3 +60,26 @@ def test_coefficients_on_the_device_are_the_hosts(lib, n, n_sys, n_v, k, prec):
         np.testing.assert_array_equal(slim["rho"], out[0]["rho"])
     finally:
         ctx.close()
+
+
+@pytest.mark.parametrize("betas", [[14.0], [0.5, 11.0, 14.0, 18.0]])
+@pytest.mark.parametrize("passes", ["store", "recompute"])
+def test_gram_of_vectors_with_subnormal_weight(lib, betas, passes):
+    """A diagonal H on basis vectors: psi_l is exp(-beta (E_l - E0) / 2) in one place, which runs
+    through float32's subnormal numbers and out below them; the Gram of each vector is its
+    square, within float32's spacing there (2^-149, half of it for each of two roundings) and
+    the float32 rounding of the coefficient above."""
+    spec = W.long_range_tfim(10, 0, 1.0, 0.0)
+    ctx = lib.Context(0)
+    try:
+        ham = lib.Hamiltonian(ctx, spec)
+        out = ham.estimate(betas, 1024, 1, 5, precision="fp32", dist="basis", full=True, passes=passes)
+        e = out["t_a"][:, 0, 0, 0]
+        subnormal = 0
+        for bi, beta in enumerate(betas):
+            psi = np.exp(-0.5 * beta * (e - e.min()))
+            subnormal += int(np.sum((psi < 2.0 ** -126) & (psi > 2.0 ** -149)))
+            np.testing.assert_array_less(np.abs(np.sqrt(out["gram_l"][bi, :, 0, 0]) - psi), 2.0 ** -149 + 4e-7 * psi)
+        assert subnormal >= 10
+    finally:
+        ctx.close()
