@@ -1436,7 +1436,9 @@ class EstimateRun {
       : ham(ham_), hm(ham_->model), s(s_), betas(betas_), n_beta(n_beta_), n_v(n_v_), k(k_), seed(seed_),
         o(o_), out(out_), prof(prof_) {}
   rdm_status prepare(char* ws, size_t ws_bytes);
-  rdm_status pass1();
+  // on: the stream of the launches (s, or one forked from it); graph: a recording may be
+  // replayed or made
+  rdm_status pass1(cudaStream_t on, bool graph);
   rdm_status finish();  // fetch_t, every dense_task, finish_rest
   // finish() in stages, so a batch can run the dense steps of all its items in one
   // parallel pass: fetch_t copies T back; dense_task(r) is recurrence r's small dense step
@@ -1463,9 +1465,10 @@ class EstimateRun {
   // Before prepare(): the first pass may run in clusters (k_pass1_cluster); after it,
   // whether it does.
   bool in_clusters = false;
-  // float32 blocks of the tiled SpMM: their own launches are faster than the packed
-  // launch's untiled units (N = 15, 16 of the serving mix: a burst of 24 requests, N 12-16,
-  // 206 -> 131 ms).
+  // float32 blocks of the tiled SpMM (from 32 tiles): their own launches, side by side with
+  // other items', are faster than the packed launch's untiled units at every size measured,
+  // least so for many items of one slice: 40 of 32 tiles (N = 15) 15.9 against 22.6 ms for
+  // d_s = 2 and 24.2 against 32.2 for d_s = 4; 16 of 128 tiles 11.3 against 26.7.
   bool tiled_launches() const { return sa.tile_k != nullptr && !in_clusters && L.precision == RDM_FP32; }
 
  private:
@@ -1577,6 +1580,29 @@ struct SideStream {
     if (stream) cudaStreamDestroy(stream);  // (its work completes first)
   }
 };
+using SideStreams = std::array<SideStream, 7>;
+
+// The first n of `side` forked from s, and joined to it again.
+static rdm_status fork_all(SideStreams& side, int n, cudaStream_t s) {
+  for (int w = 0; w < n; ++w)
+    if (side[w].fork(s) != cudaSuccess) {
+      set_error("batch: no side stream: %s", cudaGetErrorString(cudaGetLastError()));
+      return RDM_ECUDA;
+    }
+  return RDM_OK;
+}
+static rdm_status join_all(SideStreams& side, int n, cudaStream_t s) {
+  rdm_status st = RDM_OK;
+  for (int w = 0; w < n; ++w) {
+    if (!side[w].open) continue;  // (its fork failed)
+    const cudaError_t e = side[w].join(s);
+    if (e != cudaSuccess && st == RDM_OK) {
+      set_error("batch: %s", cudaGetErrorString(e));
+      st = RDM_ECUDA;
+    }
+  }
+  return st;
+}
 // Estimates whose blocks have fewer 1024-state tiles (all slices together) run the plain
 // SpMM (rdm_set_spmm_form).
 constexpr int64_t kTiledMinTiles = 32;
@@ -1731,7 +1757,7 @@ PackedItem EstimateRun::packed_item() const {
   return it;
 }
 
-rdm_status EstimateRun::pass1() {
+rdm_status EstimateRun::pass1(cudaStream_t on, bool graph) {
   rdm_status st = RDM_OK;
   // k steps; `launch` false only walks the buffer rotation (the launches are replayed
   // from a graph).
@@ -1764,12 +1790,13 @@ rdm_status EstimateRun::pass1() {
     }
     return RDM_OK;
   };
-  // Graph path: not while kernels are being timed one by one, and only for handles of
-  // a context (the serving loop's per-request handles are used once).
+  // Graph path: not while kernels are being timed one by one or several items' launches are
+  // in flight (a handle's recording may be replaced), and only for handles of a context (the
+  // serving loop's per-request handles are used once).
   bool replayed = false;
   Pass1Graph& pg = ham->graph;
   std::unique_lock<std::mutex> glk(pg.mu, std::defer_lock);
-  if (ham->ctx && ham->ctx->graphs && !(prof && prof->on) && glk.try_lock()) {
+  if (graph && ham->ctx && ham->ctx->graphs && !(prof && prof->on) && glk.try_lock()) {
     auto bits = [](double x) {
       uint64_t u;
       std::memcpy(&u, &x, sizeof u);
@@ -1784,11 +1811,11 @@ rdm_status EstimateRun::pass1() {
         (uint64_t)L.D, (uint64_t)L.DS, (uint64_t)L.B, (uint64_t)L.Bs, (uint64_t)L.n_slices, (uint64_t)L.VW,
         (uint64_t)L.TPR, (uint64_t)L.gridx, (uint64_t)L.precision, (uint64_t)L.elem};
     if (pg.exec && pg.key == key) {
-      CK(cudaGraphLaunch(pg.exec, s));
+      CK(cudaGraphLaunch(pg.exec, on));
       replayed = true;
     } else if (pg.seen == key) {
       // second call with this configuration: record it (on a private stream, since the
-      // legacy default stream cannot be captured), then run the recording on s
+      // legacy default stream cannot be captured), then run the recording
       pg.reset();
       if (!pg.capture) CK(cudaStreamCreateWithFlags(&pg.capture, cudaStreamNonBlocking));
       CK(cudaStreamBeginCapture(pg.capture, cudaStreamCaptureModeRelaxed));
@@ -1800,7 +1827,7 @@ rdm_status EstimateRun::pass1() {
       if (rs == RDM_OK && ce == cudaSuccess && g && cudaGraphInstantiate(&ex, g, 0) == cudaSuccess) {
         pg.exec = ex;
         pg.key = key;
-        CK(cudaGraphLaunch(pg.exec, s));
+        CK(cudaGraphLaunch(pg.exec, on));
         replayed = true;
       } else {
         cudaGetLastError();  // fall back to direct launches below
@@ -1811,7 +1838,7 @@ rdm_status EstimateRun::pass1() {
       pg.seen = key;
     }
   }
-  st = pass1(s, !replayed);
+  st = pass1(on, !replayed);
   return st;
 }
 
@@ -2357,7 +2384,7 @@ static rdm_status estimate_shards(rdm_ham* ham, cudaStream_t s, char* ws, size_t
     r.t_b = out->t_b ? out->t_b + (size_t)off * k * nvo : nullptr;
     EstimateRun run(ham, s, betas, n_beta, cnt, k, seed, &q, &r, prof);
     rdm_status st = run.prepare(ws, ws_bytes);
-    if (st == RDM_OK) st = run.pass1();
+    if (st == RDM_OK) st = run.pass1(s, true);
     if (st == RDM_OK) st = run.finish();
     if (st != RDM_OK) return st;
     e0s.push_back(r.e0);
@@ -2411,7 +2438,7 @@ rdm_status estimate_impl(rdm_ham* ham, cudaStream_t s, char* ws, size_t ws_bytes
   if (n_sh > 0) return estimate_shards(ham, s, ws, ws_bytes, betas, n_beta, n_v, k, seed, o, out, prof, n_sh);
   EstimateRun run(ham, s, betas, n_beta, n_v, k, seed, o, out, prof);
   rdm_status st = run.prepare(ws, ws_bytes);
-  if (st == RDM_OK) st = run.pass1();
+  if (st == RDM_OK) st = run.pass1(s, true);
   if (st == RDM_OK) st = run.finish();
   return st;
 }
@@ -2589,7 +2616,7 @@ static rdm_status run_clusters(cudaStream_t s, const std::vector<EstimateRun*>& 
     return ((int64_t)x->k * x->n_slices << x->c_log) > ((int64_t)y->k * y->n_slices << y->c_log);
   });
   const bool timing = prof && prof->on;
-  std::array<SideStream, 3> side;
+  std::array<SideStream, 7> side;
   int n_side = 0;
   rdm_status st = RDM_OK;
   for (size_t q = 0; q < order.size() && st == RDM_OK; ++q) {
@@ -2709,11 +2736,31 @@ rdm_status estimate_batch_impl(rdm_ctx* ctx, cudaStream_t s, char* ws, size_t ws
       for (int i : idx) items[i].status = items[i].status == RDM_OK ? RDM_OK : items[i].status;
       for (int i : idx) runs[i]->packed_done = true;
     }
-  // first passes of the other items, then every item's T back to the host
+  // First passes of the other items, side by side on a few streams: an item of few tiles
+  // fills a part of the GPU and is bound by its launches' latency. One after another, with a
+  // host wait each, 40 items of one slice (N = 15, d_s = 4) took 91 ms where the packed launch
+  // took 32; on 4 streams 34.8, on 6 28.0, on 8 24.2. Then every item's T back to the host.
+  {
+    std::vector<int> own;
+    for (int i = 0; i < n; ++i)
+      if (items[i].status == RDM_OK && !runs[i]->packed_done) own.push_back(i);
+    SideStreams side;
+    const int n_side = prof && prof->on ? 0 : (int)std::min(side.size(), own.empty() ? 0 : own.size() - 1);
+    rdm_status st = fork_all(side, n_side, s);
+    for (size_t q = 0; q < own.size(); ++q) {
+      const size_t w = n_side ? q % (n_side + 1) : 0;
+      if (st == RDM_OK) items[own[q]].status = runs[own[q]]->pass1(w ? side[w - 1].stream : s, own.size() == 1);
+    }
+    const rdm_status sj = join_all(side, n_side, s);
+    if (st == RDM_OK) st = sj;
+    for (int i : own) {
+      if (st != RDM_OK) items[i].status = st;
+      if (items[i].status != RDM_OK && first_bad == RDM_OK) first_bad = items[i].status;
+    }
+  }
   for (int i = 0; i < n; ++i) {
     if (items[i].status != RDM_OK) continue;
-    rdm_status st = runs[i]->packed_done ? RDM_OK : runs[i]->pass1();
-    if (st == RDM_OK) st = runs[i]->fetch_t();
+    const rdm_status st = runs[i]->fetch_t();
     items[i].status = st;
     if (st != RDM_OK && first_bad == RDM_OK) first_bad = st;
   }

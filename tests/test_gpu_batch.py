@@ -197,3 +197,34 @@ def test_batch_first_passes_in_clusters(lib, n, n_sys):
             np.testing.assert_allclose(a["rho"], a["rho_quad"], atol=1e-4, rtol=0)
     finally:
         ctx.close()
+
+
+@pytest.mark.parametrize("n,n_sys,n_v", [(15, 2, 2), (15, 1, 4), (16, 2, 2)])
+def test_many_small_items_are_no_slower_than_the_packed_launch(lib, n, n_sys, n_v):
+    """Items of 32 tiles and up run their first passes by their own launches, side by side: 24
+    of them of one slice each take no longer than in the packed launch (a quarter more is the
+    margin for the clock), and each gives what it gives alone, bit for bit."""
+    import time
+    ctx = lib.Context(0)
+    try:
+        jobs = [dict(ham=lib.Hamiltonian(ctx, W.xxz_chain(n, n_sys, 1.0, 0.3 + 0.02 * i, 0.1)), betas=[1.0], n_v=n_v,
+                     k=20, seed=i, precision="fp32") for i in range(24)]
+        ms = []
+        for form in (0, 1, 2):
+            ctx.set_packed_form(form)
+            best = 1e9
+            for _ in range(6):
+                t0 = time.perf_counter()
+                out = ctx.estimate_batch(jobs, full=True)
+                best = min(best, time.perf_counter() - t0)
+            ms.append(1e3 * best)
+            if form == 0:
+                mix = out
+        assert ms[0] < 1.25 * min(ms[1:]), ms
+        ctx.set_packed_form(0)
+        for jb, a in list(zip(jobs, mix))[::6]:
+            alone = ctx.estimate_batch([jb], full=True)[0]
+            for key in ("rho", "lnZ", "gram_l", "t_a", "t_b"):
+                np.testing.assert_array_equal(a[key], alone[key])
+    finally:
+        ctx.close()
