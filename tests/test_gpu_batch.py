@@ -228,3 +228,23 @@ def test_many_small_items_are_no_slower_than_the_packed_launch(lib, n, n_sys, n_
                 np.testing.assert_array_equal(a[key], alone[key])
     finally:
         ctx.close()
+
+
+def test_plain_spmm_form_holds_in_batches(lib):
+    """rdm_set_spmm_form(2) asks for the plain SpMM: a batch's small float32 items then run the
+    packed launch's plain units (bit for bit those of rdm_set_packed_form(1)), not the tiled
+    arithmetic of the clusters."""
+    ctx = lib.Context(0)
+    try:
+        jobs = [dict(ham=lib.Hamiltonian(ctx, W.random_model(n, 1, n)), betas=[0.5], n_v=3, k=6, seed=9,
+                     precision="fp32") for n in (10, 12, 13)]
+        ctx.set_packed_form(1)
+        units = ctx.estimate_batch(jobs, full=True)
+        ctx.set_packed_form(0)
+        ctx.set_spmm_form(2)
+        plain = ctx.estimate_batch(jobs, full=True)
+        for a, b in zip(units, plain):
+            for key in ("rho", "t_a", "t_b"):
+                np.testing.assert_array_equal(a[key], b[key])
+    finally:
+        ctx.close()
