@@ -24,6 +24,8 @@
 #include <stdint.h>
 
 #include <algorithm>
+#include <array>
+#include <map>
 #include <mutex>
 #include <set>
 #include <type_traits>
@@ -3067,32 +3069,75 @@ cudaError_t launch_pass1_local(int precision, int ds, const PackedPlan& pp, int 
   return cudaLaunchKernel(fn, dim3((unsigned)grid), dim3(kThreads), args, smem, st);
 }
 
+// One launch of k_pass1_cluster<DS>: `at` is its attribute storage.
+template <int DS>
+static cudaError_t cluster_launch(int c_log, int n_slices, size_t smem, cudaStream_t st, cudaLaunchAttribute* at,
+                                  cudaLaunchConfig_t* cfg) {
+  const void* fn = reinterpret_cast<const void*>(k_pass1_cluster<DS>);
+  cudaError_t e = opt_in_smem(fn);
+  // (16 blocks exceed the portable cluster size)
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  *cfg = cudaLaunchConfig_t{};
+  cfg->gridDim = dim3((unsigned)n_slices << c_log);
+  cfg->blockDim = dim3(kClusterThreads);
+  cfg->dynamicSmemBytes = smem;
+  cfg->stream = st;
+  at->id = cudaLaunchAttributeClusterDimension;
+  at->val.clusterDim.x = 1u << c_log;
+  at->val.clusterDim.y = at->val.clusterDim.z = 1;
+  cfg->attrs = at;
+  cfg->numAttrs = 1;
+  return e;
+}
+
+// More than any item of up to 2^14 states needs (about 80 KB).
+constexpr size_t kClusterSmemMax = (size_t)96 * 1024;
+
+// Whether the device can hold a cluster of 2^c_log blocks of k_pass1_cluster<ds> (a device
+// partition of few SMs, or no device, cannot); asked once per device, d_s and size.
+static bool device_takes_cluster(int ds, int c_log) {
+  static std::mutex mu;
+  static std::map<std::array<int, 3>, bool> known;
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  std::lock_guard<std::mutex> lk(mu);
+  const std::array<int, 3> key{dev, ds, c_log};
+  const auto f = known.find(key);
+  if (f != known.end()) return f->second;
+  auto ask = [&](auto d) -> bool {
+    constexpr int DS = decltype(d)::value;
+    cudaLaunchAttribute at{};
+    cudaLaunchConfig_t cfg;
+    int n = 0;
+    cudaError_t e = cluster_launch<DS>(c_log, 1, kClusterSmemMax, nullptr, &at, &cfg);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&n, k_pass1_cluster<DS>, &cfg);
+    if (e != cudaSuccess) cudaGetLastError();
+    return e == cudaSuccess && n > 0;
+  };
+  const bool ok = ds == 1   ? ask(std::integral_constant<int, 1>{})
+                  : ds == 2 ? ask(std::integral_constant<int, 2>{})
+                            : ask(std::integral_constant<int, 4>{});
+  known[key] = ok;
+  return ok;
+}
+
 bool pass1_cluster_fits(const Layout& L, const TiledTerms& tt) {
-  return L.precision == RDM_FP32 && layout_tiled(L) && tt.ready && L.n_bits - kTileBits <= kClusterMaxLog &&
-         cluster_smem_bytes(tt) <= (size_t)200 * 1024;
+  const int c_log = L.n_bits - kTileBits;
+  return L.precision == RDM_FP32 && layout_tiled(L) && tt.ready && c_log <= kClusterMaxLog &&
+         cluster_smem_bytes(tt) <= kClusterSmemMax && device_takes_cluster(L.DS, c_log);
 }
 
 cudaError_t launch_pass1_cluster(int ds, const PackedPlan& pp, int c_log, int n_slices, size_t smem, cudaStream_t st) {
   if (c_log < 0 || c_log > kClusterMaxLog) return cudaErrorInvalidValue;
   auto go = [&](auto d) -> cudaError_t {
     constexpr int DS = decltype(d)::value;
-    const void* fn = reinterpret_cast<const void*>(k_pass1_cluster<DS>);
-    cudaError_t e = opt_in_smem(fn);
-    // (16 blocks exceed the portable cluster size)
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (e != cudaSuccess) return e;
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3((unsigned)n_slices << c_log);
-    cfg.blockDim = dim3(kClusterThreads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
     cudaLaunchAttribute at{};
-    at.id = cudaLaunchAttributeClusterDimension;
-    at.val.clusterDim.x = 1u << c_log;
-    at.val.clusterDim.y = at.val.clusterDim.z = 1;
-    cfg.attrs = &at;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_pass1_cluster<DS>, pp, c_log);
+    cudaLaunchConfig_t cfg;
+    const cudaError_t e = cluster_launch<DS>(c_log, n_slices, smem, st, &at, &cfg);
+    return e == cudaSuccess ? cudaLaunchKernelEx(&cfg, k_pass1_cluster<DS>, pp, c_log) : e;
   };
   if (ds == 1) return go(std::integral_constant<int, 1>{});
   if (ds == 2) return go(std::integral_constant<int, 2>{});

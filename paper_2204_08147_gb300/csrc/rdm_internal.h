@@ -324,8 +324,8 @@ cudaError_t launch_pass1_packed(int precision, int ds, const PackedPlan& pp, int
 cudaError_t launch_pass1_local(int precision, int ds, const PackedPlan& pp, int grid, size_t smem,
                                cudaStream_t st);
 // The first pass with one thread-block cluster per slice (k_pass1_cluster; float32, tiled
-// layouts of up to 2^14 states): whether an item can take it, the dynamic shared memory it
-// needs, and the launch over the items' n_slices slices (pre_slices; all items 2^c_log tiles
+// layouts of up to 2^14 states): whether an item can take it on this device, the dynamic
+// shared memory it needs, and the launch over the items' n_slices slices (pre_slices; all items 2^c_log tiles
 // per slice; their starting blocks, tile_k tables and M_1 ready).
 bool pass1_cluster_fits(const Layout& L, const TiledTerms& tt);
 size_t pass1_cluster_smem(const TiledTerms& tt);
