@@ -729,8 +729,8 @@ static size_t plan_bytes(const Plan& p) {
 // dense: plan room for the device small dense step if it fits the recurrences.
 static rdm_status make_plan_impl(const HostModel& hm, int n_beta, int n_v, int k, const rdm_opts* o,
                                  size_t avail, Plan* out, double beta_max, bool dense) {
-  if (n_beta < 1 || n_v < 1 || n_v > 4096 || k < 1 || k > 512) {
-    set_error("need n_beta >= 1, 1 <= n_v <= 4096, 1 <= k <= 512 (got %d, %d, %d)", n_beta, n_v, k);
+  if (n_beta < 1 || n_v < 1 || n_v > 4096 || k < 1 || k > kMaxSteps) {
+    set_error("need n_beta >= 1, 1 <= n_v <= 4096, 1 <= k <= %d (got %d, %d, %d)", kMaxSteps, n_beta, n_v, k);
     return RDM_EINVAL;
   }
   if (o->recurrence != RDM_BLOCK && o->recurrence != RDM_SINGLE) {
@@ -2445,12 +2445,29 @@ rdm_status estimate_impl(rdm_ham* ham, cudaStream_t s, char* ws, size_t ws_bytes
 
 // ---------------------------------------------------------------- batches
 
-// Bytes at the front of a batch workspace for one packed launch's descriptors (items,
-// step and prefix tables, barrier words).
-static size_t packed_meta_bytes(int n_items, int k_max) {
+// Bytes of one launch's descriptors (items, step and prefix tables, barrier words).
+static constexpr size_t packed_meta_bytes(int n_items, int k_max) {
   return ((sizeof(PackedItem) * (size_t)n_items + sizeof(int) * ((size_t)k_max + 2 + 3 * ((size_t)n_items + 1)) +
            64 + 255) / 256) * 256;
 }
+
+// Bytes at the front of a batch workspace for the descriptors of all its launches: at most
+// kBatchLaunches (a cluster launch per d_s and tiles per slice, a packed launch per precision
+// and d_s), which part the items but have a table of steps each.
+constexpr int kBatchLaunches = 3 * (kClusterMaxLog + 1) + 6;
+static constexpr size_t batch_meta_bytes(int n_items, int k_max) { return 6 * packed_meta_bytes(n_items, k_max); }
+// The largest sum of the launches' descriptors: every launch with the largest k and its size
+// rounded up by all it can be.
+static constexpr bool batch_meta_holds() {
+  for (int n = 1; n <= 4 * kBatchLaunches; ++n)  // beyond, six times an item's bytes outgrow one item's
+    for (int k = 1; k <= kMaxSteps; ++k) {
+      const size_t launches = n < kBatchLaunches ? n : kBatchLaunches;
+      const size_t sum = (size_t)n * (sizeof(PackedItem) + 3 * sizeof(int)) + launches * (packed_meta_bytes(0, k) + 255);
+      if (sum > batch_meta_bytes(n, k)) return false;
+    }
+  return true;
+}
+static_assert(batch_meta_holds(), "descriptors of a batch's launches");
 
 // One packed launch for the items `idx` of `runs` (same precision and d_s), with the
 // grid chosen by the autotuner. meta: device scratch of packed_meta_bytes.
@@ -2670,12 +2687,12 @@ rdm_status estimate_batch_impl(rdm_ctx* ctx, cudaStream_t s, char* ws, size_t ws
                                rdm_batch_item* items, int n, const size_t* need, Profiler* prof) {
   std::vector<std::unique_ptr<EstimateRun>> runs(n);
   size_t off = 0;
-  // descriptors of at most two packed launches (float32 / float64 times d_s) go first
+  // the launches' descriptors go first, then those of the device small dense step
   int k_max = 1;
   for (int i = 0; i < n; ++i) k_max = std::max(k_max, items[i].k);
-  const size_t meta_b = packed_meta_bytes(n, k_max);
+  const size_t meta_b = batch_meta_bytes(n, k_max);
   char* meta = ws;
-  off = 6 * meta_b + dense_jobs_bytes(n);
+  off = meta_b + dense_jobs_bytes(n);
   rdm_status first_bad = RDM_OK;
   bool clusters = true;  // (a packed_form other than 0 asks for the untiled units)
   if (ctx) {
@@ -2691,8 +2708,8 @@ rdm_status estimate_batch_impl(rdm_ctx* ctx, cudaStream_t s, char* ws, size_t ws
     off += need[i];
     if (it.status != RDM_OK && first_bad == RDM_OK) first_bad = it.status;
   }
-  // First passes in clusters, and the others packed, one launch per (precision, d_s). The
-  // descriptors of all groups take less than the 6 meta_b: the groups part the items.
+  // First passes in clusters, and the others packed, one launch per (precision, d_s); their
+  // descriptors follow one another in meta (batch_meta_holds).
   size_t meta_off = 0;
   std::vector<std::vector<char>> keep;
   {
@@ -2766,7 +2783,7 @@ rdm_status estimate_batch_impl(rdm_ctx* ctx, cudaStream_t s, char* ws, size_t ws
   }
   // the device small dense steps of all items that take it: one launch per d_s over all
   // their recurrences
-  char* dense_meta = ws + 6 * meta_b;
+  char* dense_meta = ws + meta_b;
   for (int ds : {1, 2, 4}) {
     std::vector<DenseJob> jobs;
     std::vector<int> idx;
@@ -2820,7 +2837,7 @@ rdm_status estimate_batch_impl(rdm_ctx* ctx, cudaStream_t s, char* ws, size_t ws
 size_t batch_workspace_bytes(const rdm_batch_item* items, int n, const size_t* avail, size_t* need) {
   int k_max = 1;
   for (int i = 0; i < n; ++i) k_max = std::max(k_max, items[i].k);
-  size_t tot = 6 * packed_meta_bytes(n, k_max) + dense_jobs_bytes(n);
+  size_t tot = batch_meta_bytes(n, k_max) + dense_jobs_bytes(n);
   for (int i = 0; i < n; ++i) {
     rdm_status st = RDM_OK;
     need[i] = estimate_bytes(items[i].ham->model, items[i].n_beta, items[i].n_v, items[i].k, &items[i].opts,

@@ -2485,7 +2485,6 @@ __global__ void __launch_bounds__(kThreads) k_pass1_local(PackedPlan pp) {
 // k_pass1_packed on items of 2^10 .. 2^14 states, which read every partner row from L2: the
 // first passes of 48 small solves (N 8-14) take 44 instead of 87 ms.
 constexpr int kClusterThreads = kConsumerWarps * 32;
-constexpr int kClusterMaxLog = 4;  // up to 16 blocks (N = 14)
 
 __device__ __forceinline__ void cluster_sync() {
   asm volatile("barrier.cluster.arrive.release;\nbarrier.cluster.wait.acquire;\n" ::: "memory");

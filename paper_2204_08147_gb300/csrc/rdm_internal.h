@@ -59,6 +59,7 @@ struct Layout {
   RDM_HD size_t block_bytes() const { return (size_t)D * (size_t)B * (size_t)elem; }
 };
 
+constexpr int kMaxSteps = 512;  // k of an estimate
 constexpr int kThreads = 256;
 
 // Number of float64 reduction values per bath-vector group for each kernel kind.
@@ -327,6 +328,7 @@ cudaError_t launch_pass1_local(int precision, int ds, const PackedPlan& pp, int 
 // layouts of up to 2^14 states): whether an item can take it on this device, the dynamic
 // shared memory it needs, and the launch over the items' n_slices slices (pre_slices; all items 2^c_log tiles
 // per slice; their starting blocks, tile_k tables and M_1 ready).
+constexpr int kClusterMaxLog = 4;  // up to 16 blocks (N = 14)
 bool pass1_cluster_fits(const Layout& L, const TiledTerms& tt);
 size_t pass1_cluster_smem(const TiledTerms& tt);
 cudaError_t launch_pass1_cluster(int ds, const PackedPlan& pp, int c_log, int n_slices, size_t smem, cudaStream_t st);

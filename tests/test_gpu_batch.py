@@ -248,3 +248,21 @@ def test_plain_spmm_form_holds_in_batches(lib):
                 np.testing.assert_array_equal(a[key], b[key])
     finally:
         ctx.close()
+
+
+def test_batch_of_every_launch(lib):
+    """One item for each launch a batch can have (clusters by d_s and size, packed launches by
+    precision and d_s), with many steps each: the launches' descriptors lie one behind the
+    other, and every item gives what it gives alone, bit for bit."""
+    ctx = lib.Context(0)
+    try:
+        jobs = [dict(ham=lib.Hamiltonian(ctx, W.long_range_tfim(n, s, 1.5, 0.9)), betas=[0.7], n_v=2, k=60 + 5 * s + n,
+                     seed=n, precision=p) for s in (0, 1, 2)
+                for n, p in ((10, "fp32"), (11, "fp32"), (12, "fp32"), (13, "fp32"), (14, "fp32"), (8, "fp32"), (9, "fp64"))]
+        mix = ctx.estimate_batch(jobs, full=True)
+        for jb, a in zip(jobs, mix):
+            alone = ctx.estimate_batch([jb], full=True)[0]
+            for key in ("rho", "lnZ", "gram_l", "t_a", "t_b"):
+                np.testing.assert_array_equal(a[key], alone[key])
+    finally:
+        ctx.close()
