@@ -679,12 +679,13 @@ struct Plan {
   int vstride;                        // its Chebyshev degree bound + 1
 };
 
-// Float64 counts of the arrays whose size depends on the grouping: reduction partials
-// (8 slots: one per beta of a stored-basis Gram launch), the E coefficients of a beta
-// chunk and the Gram results of a chunk, each
-// large enough for the recurrences' layout and for the Gram view.
+// Float64 counts of the arrays whose size depends on the grouping: reduction partials (the
+// recurrences' kernels take one grid's at a time, the Gram kernels gram1 for each beta of a
+// launch, as many betas as there is room for), the E coefficients of a beta chunk and the
+// Gram results of a chunk, each large enough for the recurrences' layout and for the Gram
+// view.
 struct PlanSizes {
-  size_t partials, e, gram;
+  size_t partials, gram1, e, gram;
 };
 static PlanSizes plan_sizes(const Plan& p) {
   const Layout& L = p.L;
@@ -692,9 +693,10 @@ static PlanSizes plan_sizes(const Plan& p) {
   const size_t rec = (size_t)L.n_groups() * L.DS * L.DS, view = (size_t)G.n_groups() * G.DS * G.DS;
   // (the packed first pass runs the untiled grid on a tiled layout: room for both)
   const size_t prec = (size_t)L.n_slices * std::max(L.gridx, untiled_gridx(L)) * L.groups_per_slice() * L.DS * L.DS;
-  const size_t pview = (size_t)G.n_slices * G.gridx * G.groups_per_slice() * G.DS * G.DS;
-  return PlanSizes{std::max(prec, pview) * 8, (size_t)p.k * p.nbc * std::max(rec, view),
-                   (size_t)p.nbc * std::max(rec, view)};
+  const size_t per_block = (size_t)G.n_slices * G.groups_per_slice() * G.DS * G.DS;
+  const size_t gram1 = per_block * gram_gridx(G);
+  return PlanSizes{std::max(gram1, 8 * std::max(prec, per_block * G.gridx)), gram1,
+                   (size_t)p.k * p.nbc * std::max(rec, view), (size_t)p.nbc * std::max(rec, view)};
 }
 
 static size_t plan_bytes(const Plan& p) {
@@ -1666,7 +1668,7 @@ rdm_status EstimateRun::prepare(char* ws, size_t ws_bytes) {
   psi = store ? nullptr
               : ar.take<char>(L.block_bytes() / (size_t)L.n_slices * (size_t)(p.nsc ? p.nsc : L.n_slices) * p.nbc);
   psz = plan_sizes(p);
-  pstride_g = (size_t)Lgr.n_slices * Lgr.gridx * Lgr.groups_per_slice() * nvo;
+  pstride_g = psz.gram1;
   partials = ar.take<double>(psz.partials);
   coef = ar.take<double>((size_t)(k + 2) * ng * nv * 3);
   d_ta = ar.take<double>((size_t)k * ng * nv);
@@ -2078,10 +2080,10 @@ rdm_status EstimateRun::finish_rest() {
     return last;
   };
   std::vector<int> jlast((size_t)p.nbc * n_v, 1), kbeta(p.nbc, 1);
-  // betas of one Gram launch: their partials fit the buffer, the launches are even
+  // betas of one Gram launch: their partials fit the buffer (one beta's do: plan_sizes; a
+  // group of slices takes less than the whole), the launches are even
   auto gram_betas = [&](size_t stride, int nb) {
-    const int slots =
-        (int)std::min<size_t>(kGramLaunchBetas, std::max<size_t>(1, psz.partials / std::max<size_t>(1, stride)));
+    const int slots = (int)std::min<size_t>(kGramLaunchBetas, psz.partials / stride);
     const int launches = (nb + slots - 1) / slots;
     return (nb + launches - 1) / launches;
   };
