@@ -2634,10 +2634,11 @@ static rdm_status run_clusters(cudaStream_t s, const std::vector<EstimateRun*>& 
   std::stable_sort(order.begin(), order.end(), [](const Group* x, const Group* y) {
     return ((int64_t)x->k * x->n_slices << x->c_log) > ((int64_t)y->k * y->n_slices << y->c_log);
   });
-  const bool timing = prof && prof->on;
-  std::array<SideStream, 7> side;
-  int n_side = 0;
-  rdm_status st = RDM_OK;
+  // Forked before the first launch: the side streams wait for what s holds now (the items'
+  // starting blocks), not for that launch.
+  SideStreams side;
+  const int n_side = prof && prof->on ? 0 : (int)std::min(side.size(), order.size() - 1);
+  rdm_status st = fork_all(side, n_side, s);
   for (size_t q = 0; q < order.size() && st == RDM_OK; ++q) {
     Group& g = *order[q];
     // (launches of items with different k do not need the k-sorted order of the packed grid)
@@ -2647,19 +2648,7 @@ static rdm_status run_clusters(cudaStream_t s, const std::vector<EstimateRun*>& 
     std::memcpy(img.data() + o_pre, g.pre.data(), sizeof(int) * g.pre.size());
     char* dev = meta + *used;
     *used += packed_meta_bytes((int)g.items.size(), g.k);
-    cudaStream_t ls = s;
-    if (!timing && q > 0) {
-      const int w = (int)((q - 1) % side.size());
-      if (w >= n_side) {
-        if (side[w].fork(s) != cudaSuccess) {
-          set_error("batch: no side stream: %s", cudaGetErrorString(cudaGetLastError()));
-          st = RDM_ECUDA;
-          break;
-        }
-        n_side = w + 1;
-      }
-      ls = side[w].stream;
-    }
+    cudaStream_t ls = n_side && q > 0 ? side[(q - 1) % n_side].stream : s;
     PackedPlan pp{};
     pp.items = reinterpret_cast<const PackedItem*>(dev);
     pp.n_items = (int)g.items.size();
@@ -2675,14 +2664,8 @@ static rdm_status run_clusters(cudaStream_t s, const std::vector<EstimateRun*>& 
       st = RDM_ECUDA;
     }
   }
-  for (int w = 0; w < n_side; ++w) {
-    const cudaError_t e = side[w].join(s);
-    if (e != cudaSuccess && st == RDM_OK) {
-      set_error("batch: %s", cudaGetErrorString(e));
-      st = RDM_ECUDA;
-    }
-  }
-  return st;
+  const rdm_status sj = join_all(side, n_side, s);
+  return st != RDM_OK ? st : sj;
 }
 
 rdm_status estimate_batch_impl(rdm_ctx* ctx, cudaStream_t s, char* ws, size_t ws_bytes,

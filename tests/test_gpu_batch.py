@@ -266,3 +266,39 @@ def test_batch_of_every_launch(lib):
                 np.testing.assert_array_equal(a[key], alone[key])
     finally:
         ctx.close()
+
+
+def test_cluster_launches_run_side_by_side(lib):
+    """Four items of one slice each, of four sizes: four cluster launches, which take a fraction
+    of the GPU each and run at the same time. Timed launches (the profile) run one after
+    another; untimed, the batch takes that less the sum of their times, and the longest of
+    them more (with half of that as the margin)."""
+    import time
+    ctx = lib.Context(0)
+    try:
+        jobs = [dict(ham=lib.Hamiltonian(ctx, W.long_range_xxz(n, 0, 1.0, 0.8)), betas=[0.5], n_v=1, k=400, seed=3,
+                     precision="fp32") for n in (10, 11, 12, 13)]
+
+        def clock(batch):
+            best = 1e9
+            for _ in range(8):
+                t0 = time.perf_counter()
+                ctx.estimate_batch(batch)
+                best = min(best, time.perf_counter() - t0)
+            return 1e3 * best
+
+        def first_pass(batch):
+            ctx.profile(True)
+            ctx.estimate_batch(batch)
+            ms = ctx.profile_stats()["packed_pass1"]["ms"]
+            ctx.profile(False)
+            return ms
+
+        clock(jobs)
+        each = [first_pass([jb]) for jb in jobs]
+        ctx.profile(True)
+        serial = clock(jobs)
+        ctx.profile(False)
+        assert clock(jobs) < serial - sum(each) + 1.5 * max(each), (serial, each)
+    finally:
+        ctx.close()
