@@ -742,15 +742,24 @@ __device__ __forceinline__ void reg_uniform(T (&y)[RPT][VW], const T (&x)[RPT][V
   if (in_use(c_even)) reg_half<K, 0>(y, x, c_even);
   if (in_use(c_odd)) reg_half<K, 1>(y, x, c_odd);
 }
-// ... or differ between its lanes (a half is skipped when it is zero on all of them).
-template <int K, typename T, int VW, int RPT>
+// Whether a thread takes part in a term whose coefficient c may differ between the lanes of
+// its warp. The recurrences' lanes all do where one of them needs it (a zero coefficient on
+// the others), rather than diverge. H x of a caller's x (EXACT) leaves out the rows whose
+// coefficient is zero: x may hold infinities or NaN, and 0 * x would put them into rows that H
+// does not couple to theirs.
+template <bool EXACT, typename T>
+__device__ __forceinline__ bool lane_takes(T c) {
+  return EXACT ? in_use(c) : __any_sync(0xffffffffu, in_use(c)) != 0;
+}
+// ... or differ between its lanes.
+template <int K, bool EXACT, typename T, int VW, int RPT>
 __device__ __forceinline__ void reg_lanes(T (&y)[RPT][VW], const T (&x)[RPT][VW], T c_even, T c_odd) {
-  if (__any_sync(0xffffffffu, in_use(c_even))) reg_half<K, 0>(y, x, c_even);
-  if (__any_sync(0xffffffffu, in_use(c_odd))) reg_half<K, 1>(y, x, c_odd);
+  if (lane_takes<EXACT>(c_even)) reg_half<K, 0>(y, x, c_even);
+  if (lane_takes<EXACT>(c_odd)) reg_half<K, 1>(y, x, c_odd);
 }
 
 // The in-tile terms: y += (terms) x, xo the thread's own rows of the tile `own`.
-template <bool UNI, int RG, int STEP, typename T, int VW, int RPT>
+template <bool UNI, bool EXACT, int RG, int STEP, typename T, int VW, int RPT>
 __device__ __forceinline__ void own_terms(T (&y)[RPT][VW], const T (&xo)[RPT][VW], const T* own, int rgoff,
                                           const TiledTerms& tt, const T* s_reg, const GrpS<T>* grp,
                                           const LaneS<T>* lanet, uint32_t act_lane, uint32_t act_grp) {
@@ -780,9 +789,9 @@ __device__ __forceinline__ void own_terms(T (&y)[RPT][VW], const T (&xo)[RPT][VW
 #pragma unroll
       for (int m = 0; m < RPT; ++m) axpy(y[m], c, xp[m]);
     }
-    if (fl & kPatReg) reg_lanes<1>(y, xp, odd ? G.co[0] : G.ce[0], odd ? G.ce[0] : G.co[0]);
-    if (fl & (kPatReg << 1)) reg_lanes<2>(y, xp, odd ? G.co[1] : G.ce[1], odd ? G.ce[1] : G.co[1]);
-    if (fl & (kPatReg << 2)) reg_lanes<4>(y, xp, odd ? G.co[2] : G.ce[2], odd ? G.ce[2] : G.co[2]);
+    if (fl & kPatReg) reg_lanes<1, EXACT>(y, xp, odd ? G.co[0] : G.ce[0], odd ? G.ce[0] : G.co[0]);
+    if (fl & (kPatReg << 1)) reg_lanes<2, EXACT>(y, xp, odd ? G.co[1] : G.ce[1], odd ? G.ce[1] : G.co[1]);
+    if (fl & (kPatReg << 2)) reg_lanes<4, EXACT>(y, xp, odd ? G.co[2] : G.ce[2], odd ? G.ce[2] : G.co[2]);
   }
   // terms of the row-group spins alone
   if constexpr (UNI) {
@@ -795,14 +804,13 @@ __device__ __forceinline__ void own_terms(T (&y)[RPT][VW], const T (&xo)[RPT][VW
     for (int t = 0; t < tt.n_own; ++t) {
       const LaneS<T> d = lanet[t];
       const T c = ((act_lane >> t) & 1u) ? d.co : d.ce;
-      // where the coefficient differs across the warp's lanes they all run the term
-      if (__any_sync(0xffffffffu, in_use(c))) rows_fma<STEP>(y, own + (rgoff ^ (int)d.off), c);
+      if (lane_takes<EXACT>(c)) rows_fma<STEP>(y, own + (rgoff ^ (int)d.off), c);
     }
   }
 }
 // The terms of one high spin on its partner tile P: its field and its hops with in-tile
 // spins (hs: whether it is down here).
-template <bool UNI, int STEP, typename T, int VW, int RPT>
+template <bool UNI, bool EXACT, int STEP, typename T, int VW, int RPT>
 __device__ __forceinline__ void single_terms(T (&y)[RPT][VW], const T* P, int rgoff, int rg, const PatS<T>& A, bool hs,
                                              const LaneS<T>* lanet) {
   const uint32_t fl = A.flags;
@@ -822,7 +830,7 @@ __device__ __forceinline__ void single_terms(T (&y)[RPT][VW], const T* P, int rg
     const LaneS<T> d = lanet[t];
     const bool odd = (((uint32_t)rg & d.low) != 0u) != hs;
     const T c = UNI || odd ? d.co : d.ce;
-    if (UNI || __any_sync(0xffffffffu, in_use(c))) rows_fma<STEP>(y, P + (rgoff ^ (int)d.off), c);
+    if (UNI || lane_takes<EXACT>(c)) rows_fma<STEP>(y, P + (rgoff ^ (int)d.off), c);
   }
 }
 // An opposite-spin pair: term l of group A (its spin down here, tile Z) acts on the rows
@@ -1251,12 +1259,12 @@ __global__ void __launch_bounds__(kTiledThreads, 1) k_spmm_tiled(Layout L, SpmmA
 #pragma unroll
         for (int v = 0; v < VW; ++v) y[m][v] = dg[m] * xo[m][v];
     }
-    own_terms<UNI, RG, kStep>(y, xo, own, rgoff, tt, s_reg, grp, lanet, act_lane, act_grp);
+    own_terms<UNI, MODE == kModeApply, RG, kStep>(y, xo, own, rgoff, tt, s_reg, grp, lanet, act_lane, act_grp);
     release();
     // Partner tiles, in the producer's order: opposite-spin pairs, single-spin patterns, the
     // flat ones in use.
     auto single = [&](const PatS<T>& A) {
-      single_terms<UNI, kStep>(y, sp, rgoff, rg, A, (ut & A.high) != 0u, lanet);
+      single_terms<UNI, MODE == kModeApply, kStep>(y, sp, rgoff, rg, A, (ut & A.high) != 0u, lanet);
     };
     if constexpr (UNI) {
       for (int st = 0; st < n_st;) {
@@ -2604,7 +2612,7 @@ __global__ void __launch_bounds__(kClusterThreads, 2) k_pass1_cluster(PackedPlan
 #pragma unroll
         for (int v = 0; v < VW; ++v) y[m][v] = dg[m] * xo[m][v];
     }
-    own_terms<false, RG, kStep>(y, xo, cur, rgoff, tt, s_reg, grp, lanet, act_lane, act_grp);
+    own_terms<false, false, RG, kStep>(y, xo, cur, rgoff, tt, s_reg, grp, lanet, act_lane, act_grp);
     // partner tiles in the tiled SpMM's order
     uint32_t om = up_pairs, zm = ~up_pairs & (uint32_t)((1u << tt.n_pair) - 1u);
     for (int joint = min(__popc(zm), __popc(om)); zm | om; --joint) {
@@ -2618,11 +2626,11 @@ __global__ void __launch_bounds__(kClusterThreads, 2) k_pass1_cluster(PackedPlan
         const int p = __ffs((int)(zm | om)) - 1;
         zm &= ~(1u << p);
         om &= ~(1u << p);
-        single_terms<false, kStep>(y, peer(cur, rank ^ pat[p].high), rgoff, rg, pat[p], (rank & pat[p].high) != 0u, lanet);
+        single_terms<false, false, kStep>(y, peer(cur, rank ^ pat[p].high), rgoff, rg, pat[p], (rank & pat[p].high) != 0u, lanet);
       }
     }
     for (int p = tt.n_pair; p < tt.n_pair + tt.n_single; ++p)
-      single_terms<false, kStep>(y, peer(cur, rank ^ pat[p].high), rgoff, rg, pat[p], (rank & pat[p].high) != 0u, lanet);
+      single_terms<false, false, kStep>(y, peer(cur, rank ^ pat[p].high), rgoff, rg, pat[p], (rank & pat[p].high) != 0u, lanet);
     for (int p = tt.n_pair + tt.n_single; p < tt.n_part; ++p) {
       const T c = (__popc(rank & pat[p].high) & 1) ? pat[p].co[0] : pat[p].ce[0];
       if (in_use(c)) rows_fma<kStep>(y, peer(cur, rank ^ pat[p].high) + rgoff, c);
