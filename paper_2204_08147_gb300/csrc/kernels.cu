@@ -676,6 +676,21 @@ __device__ __forceinline__ bool ring_wait(uint64_t* bar, uint32_t parity, volati
   return false;
 }
 
+// At a producer's end: no copy of its may still be on its way into the ring when the block
+// ends. In a whole run the consumers have waited for all of them, but not after a wait that
+// gave up, so it waits for the last copy into each of its slots (q, q + kProducerWarps, ..),
+// bounded, and not cut short by the abort flag. slot, round: the stage after its last; the
+// stage at which it stopped was not issued. (Apart: inlined, the loop cost the transverse
+// field at N = 22 0.3%.)
+__device__ __noinline__ void drain_ring(uint64_t* full, int stages, int q, int slot, uint32_t round, bool stop) {
+  const int failed = !stop ? -1 : (slot == 0 ? stages : slot) - 1;
+  for (int sl = q; sl < stages; sl += kProducerWarps) {
+    const uint32_t copies = round + (sl < slot ? 1u : 0u) - (sl == failed ? 1u : 0u);
+    for (uint32_t it = 0; copies && it < (1u << 20) && !mbar_try_wait(&full[sl], (copies - 1u) & 1u); ++it) {
+    }
+  }
+}
+
 // Rows of a consumer thread: row rg + RG m (m = 0..RPT-1) of a tile sits at element offset
 // rgoff + m * kStep (rgoff = rg * BS + lane * VW, kStep = RG * BS). Under a mask m_low in the
 // row-group bits its partner rows sit at (rgoff ^ m_low * BS) + m * kStep: one address and
@@ -1096,7 +1111,10 @@ __global__ void __launch_bounds__(kTiledThreads, 1) k_spmm_tiled(Layout L, SpmmA
           next_stage(ut, 0, (T)0, Wp + ((size_t)ut << kTileBits) * BS, 0u, nullptr, stream);
         }
       }
-    if (stop && pl == 0) atomicOr(a.err, 1u);
+    if (pl == 0) {
+      drain_ring(full, kStages, (int)q, slot, round, stop);
+      if (stop) atomicOr(a.err, 1u);
+    }
     return;
   }
 
