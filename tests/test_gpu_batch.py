@@ -302,3 +302,23 @@ def test_cluster_launches_run_side_by_side(lib):
         assert clock(jobs) < serial - sum(each) + 1.5 * max(each), (serial, each)
     finally:
         ctx.close()
+
+
+@pytest.mark.parametrize("n,n_sys", [(13, 0), (14, 1), (14, 2)])
+@pytest.mark.parametrize("field", [0.0, 0.45])
+def test_uniform_hops_in_clusters(lib, n, n_sys, field):
+    """XX couplings of all pairs (no parity-dependent coefficient) through the cluster pass,
+    against the packed launch's plain units, within the float32 rounding of six steps."""
+    spec = W.long_range_xxz(n, n_sys, 1.2, 0.6, 0.2, 0.9)
+    spec.jy[:] = 0.0
+    spec.gx[::2] = field
+    ctx = lib.Context(0)
+    try:
+        job = dict(ham=lib.Hamiltonian(ctx, spec), betas=[0.4], n_v=5, k=6, seed=2, precision="fp32")
+        a = ctx.estimate_batch([job], full=True)[0]
+        ctx.set_packed_form(1)
+        b = ctx.estimate_batch([job], full=True)[0]
+        for key in ("t_a", "t_b"):
+            np.testing.assert_allclose(a[key], b[key], atol=2e-5 * job["ham"].info()["norm_bound"], rtol=0)
+    finally:
+        ctx.close()

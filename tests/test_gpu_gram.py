@@ -83,3 +83,29 @@ def test_gram_of_vectors_with_subnormal_weight(lib, betas, passes):
         assert subnormal >= 10
     finally:
         ctx.close()
+
+
+@pytest.mark.parametrize("n,n_sys,n_v,k,n_beta", [
+    (12, 2, 3, 80, 9),    # groups of 2 betas (their coefficients pass 36 KB at 4)
+    (12, 2, 3, 160, 3),   # groups of 1
+    (12, 1, 3, 160, 5),   # d_s = 2, groups of 2
+    (10, 0, 9, 6, 300),   # more betas than one launch takes
+    (18, 0, 1, 6, 40),    # one slice: as many betas a launch as the partials have room for
+])
+def test_gram_groups_of_long_recurrences_and_grids(lib, n, n_sys, n_v, k, n_beta):
+    """Each of a few betas of the grid gives bit for bit what it gives alone."""
+    spec = W.xxz_chain(n, n_sys, 1.0, 0.5, 0.1)
+    betas = W.beta_grid(n_beta, 0.05, 12.0)
+    ctx = lib.Context(0)
+    try:
+        ham = lib.Hamiltonian(ctx, spec)
+        ctx.set_device_dense(0)  # the same coefficients whatever the grid
+
+        def run(b):
+            return ham.estimate(b, n_v, k, 3, precision="fp32", dist="rademacher", full=True)
+        grid = run(betas)
+        for i in sorted({0, n_beta // 3, n_beta // 2, n_beta - 1}):
+            np.testing.assert_array_equal(grid["gram_l"][i], run(betas[i:i + 1])["gram_l"][0])
+        np.testing.assert_allclose(grid["rho"], grid["rho_quad"], atol=1e-4, rtol=0)
+    finally:
+        ctx.close()

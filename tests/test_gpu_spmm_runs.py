@@ -85,3 +85,34 @@ def test_apply_keeps_infinities_to_coupled_rows(lib, model, cols, dtype):
                 assert torch.isfinite(y[:, [0, 2, 3]]).all()
     finally:
         ctx.close()
+
+
+@pytest.mark.parametrize("n,n_sys,n_v,prec,tol", [
+    (13, 0, 40, "fp32", 2e-5),
+    (14, 2, 30, "fp32", 2e-5),
+    (15, 1, 9, "fp32", 2e-5),
+    (13, 1, 21, "fp64", 1e-12),
+    (14, 2, 10, "fp64", 1e-12),
+])
+@pytest.mark.parametrize("model", ["xx", "xx+x"])
+def test_uniform_hops_match_the_plain_spmm(lib, n, n_sys, n_v, prec, tol, model):
+    """XX couplings of all pairs (c_odd = c_even) take the uniform instantiation with every kind
+    of term: hops of register, row-group and high spins with one another, with and without
+    fields. A_j and B_j of five steps against the plain SpMM, and rho against the oracle."""
+    from oracle import lanczos
+    spec = _model(model, n, n_sys)
+    ctx = lib.Context(0)
+    try:
+        ham = lib.Hamiltonian(ctx, spec)
+        out = {}
+        for form in (1, 2):
+            ctx.set_spmm_form(form)
+            out[form] = ham.estimate([0.4], n_v, 5, 31, precision=prec, dist="rademacher", full=True)
+        bound = ham.info()["norm_bound"]
+        for key in ("t_a", "t_b"):
+            np.testing.assert_allclose(out[1][key], out[2][key], atol=tol * bound, rtol=0)
+        if n == 13:
+            ref = lanczos.Estimator(spec).run(np.array([0.4]), n_v, 5, 31, "rademacher")
+            np.testing.assert_allclose(out[1]["rho"], ref["rho"], atol=1e-4 if prec == "fp32" else 1e-10, rtol=0)
+    finally:
+        ctx.close()
