@@ -570,17 +570,17 @@ def serving_bench(rdm, ctx, n_req: int, n_min: int = 12, n_max: int = 18, budget
                                             "p99": 1000 * float(np.percentile(lat, 99))}}
     return {"requests": n_req, "saturated_solves_per_s": rate, "poisson": loads,
             "stream": f"XXZ/LR-TFIM mix, N {n_min}..{n_max}, N_s 1-2, 8-64 betas, n_v 8-64, k 30-100, float32; "
-                      "small requests share packed launches",
+                      "small requests run as batches",
             "max_inflight": 4, "budget_gib": budget >> 30}
 
 
 def batch_bench(rdm, ctx, n_req: int = 48) -> dict:
     """Uneven small instances (the serving stream's XXZ / LR-TFIM mix with N 8..14, N_s 1-2,
     8-64 betas, n_v 8-64, k 30-100, float32) estimated one at a time through rdm_estimate
-    and all at once through rdm_estimate_batch (their first passes in one persistent
-    cooperative launch), after one warm-up of each (the batch's warm-up runs the
-    autotuner). Host-timed around the blocking calls; the device time of the packed
-    launch and of the per-item launches comes from a profiled repeat."""
+    and all at once through rdm_estimate_batch (their first passes in clusters, or in the
+    persistent cooperative launch), after one warm-up of each (the batch's warm-up runs the
+    autotuner). Host-timed around the blocking calls; the device time of the first
+    passes and of the per-item launches comes from a profiled repeat."""
     reqs = W.serving_requests(n_req, seed=20220422, n_min=8, n_max=14)
     hams = [rdm.Hamiltonian(ctx, r["spec"]) for r in reqs]
     jobs = [dict(ham=h, betas=r["betas"], n_v=r["n_v"], k=r["k"], seed=r["seed"], precision="fp32")

@@ -318,9 +318,10 @@ typedef struct {
  *   - float32 items of 2^10 .. 2^14 states that keep their Krylov basis (k+1 blocks fit) with
  *     a block of at most 64 MB: one thread-block cluster per slice (bath vectors of one
  *     32-byte row), all steps in the clusters' shared memory, one launch per (d_s, N) over
- *     all such items;
+ *     all such items (not with rdm_set_spmm_form 2, nor on a device that cannot hold the
+ *     clusters: the packed launch then);
  *   - larger float32 items whose block the tiled SpMM takes, and items above 64 MB or with a
- *     recomputed basis: as rdm_estimate does;
+ *     recomputed basis: as rdm_estimate does, several items side by side;
  *   - the others (N < 10, float64) in ONE persistent cooperative launch with the other such
  *     items of their precision and d_s -- the SpMM, A_j, orthogonalisation and QR phases of
  *     every item, separated by grid barriers. Each work unit of that launch is one block of
@@ -364,7 +365,8 @@ rdm_status rdm_set_packed_form(rdm_ctx* ctx, int form);
  * 16 (FP64). X and Y must not overlap. Asynchronous on the context's stream,
  * except when the block takes the tiled SpMM (32-byte rows: n_cols = 8 FP32 or
  * 4 FP64, N >= 10): then the call waits for the kernel to read back its copy-ring
- * status (RDM_ECUDA if a copy wait gave up). This is the SpMM of the hot path (the
+ * status (RDM_ECUDA if a copy wait gave up). An infinity or NaN in X reaches its own row
+ * and the rows that H couples to it, no others. This is the SpMM of the hot path (the
  * matrix-vector products of Sec. 2.4), exposed for verification. */
 rdm_status rdm_apply_hamiltonian(rdm_ham* ham, int precision, const void* x, void* y,
                                  int n_cols);
