@@ -1463,7 +1463,7 @@ class EstimateRun {
   bool packable() const;
   PackedItem packed_item() const;
   const Plan& plan() const { return p; }
-  bool packed_done = false;  // the first pass ran in a packed launch
+  bool packed_done = false;  // the first pass ran in a launch shared with other items
   // Before prepare(): the first pass may run in clusters (k_pass1_cluster); after it,
   // whether it does.
   bool in_clusters = false;

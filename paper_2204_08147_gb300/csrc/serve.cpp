@@ -20,7 +20,7 @@ struct Request {
   rdm_opts opts{};
   rdm_result* out = nullptr;
   size_t footprint = 0;
-  bool packable = false;  // runs its first pass in a packed launch with other requests
+  bool packable = false;  // runs in a batch with other requests
   rdm_status status = RDM_OK;
   bool done = false;
   double t_submit = 0, t_admit = 0, t_done = 0;
@@ -28,7 +28,7 @@ struct Request {
 };
 
 struct ServeState {
-  rdm_ctx* ctx = nullptr;  // the owning context (its autotuner serves the packed launches)
+  rdm_ctx* ctx = nullptr;  // the owning context (its autotuner serves the batches' packed launches)
   int device = 0;
   size_t budget = 0, used = 0;
   int max_inflight = 1, inflight = 0;
@@ -90,8 +90,8 @@ static rdm_status run_request(ServeState& S, Request& r, cudaStream_t st) {
   return s;
 }
 
-// A batch of packable requests: their first passes share one packed launch
-// (estimate_batch_impl); each request's result is the same as when it runs alone.
+// A batch of packable requests: their first passes run together (in clusters, packed or side by
+// side: estimate_batch_impl); each request's result is the same as when it runs alone.
 static rdm_status run_batch(ServeState& S, std::vector<std::shared_ptr<Request>>& rs, cudaStream_t st,
                             std::vector<rdm_status>& status) {
   if (cudaSetDevice(S.device) != cudaSuccess) {
@@ -319,7 +319,7 @@ extern "C" rdm_status rdm_submit(rdm_ctx* ctx, const rdm_model* model, const dou
                             opts->recurrence, bmax);
   }
   if (fp == 0) return RDM_EINVAL;  // make_plan set the error
-  // Small requests keep their Krylov basis and join packed launches (rdm_estimate_batch)
+  // Small requests keep their Krylov basis and join batches (rdm_estimate_batch)
   // when that takes at most a quarter of the budget.
   if (opts->passes != RDM_PASSES_RECOMPUTE) {
     const size_t fs = packed_store_footprint(r->hm, n_beta, n_v, k, opts, bmax);
